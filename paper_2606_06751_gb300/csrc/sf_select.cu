@@ -436,53 +436,121 @@ __global__ void __launch_bounds__(kMedThreads)
 }
 
 // ---------------------------------------------------------------------------
-// Top-k.  One CTA per window.  Order: value descending, then index ascending
-// (index = stage for X, s*R + r for E); value 0 is not a suspect.
+// Top-k.  Order: value descending, then index ascending (index = stage for X,
+// s*R + r for E); value 0 is not a suspect.
+//
+// A window's (stage, rank) entries are split over a cluster of one to
+// kTopCluster CTAs (top_cluster: one tile of entries each, eight at most).  Each CTA reads its slice once, kTopTile entries at a time with the
+// next tile's loads in flight, and appends the positive entries to a list in
+// shared memory: lead-rank credit is sparse (at most one rank per step and
+// stage), so a slice's list usually ends far below its capacity.  A list that
+// could not take another whole tile is first cut to its k best.  The cut runs
+// in registers, warp by warp (k rounds of a warp arg-max, no CTA barrier
+// between rounds), then over the warps' k best; the cluster's first CTA merges
+// the CTAs' k best through distributed shared memory.  What is left is the
+// latency of one pass of loads, three cuts and two cluster barriers: k = 5 of
+// 20 windows of 8192 x 8 entries takes 14.5 us (33.2 us as k rounds of a block
+// arg-max that each re-read the slice), of one window 10.9 us (20.6 us).
 constexpr int kTopThreads = 256;
+constexpr int kTopWarps = kTopThreads / 32;
+constexpr int kTopCluster = 8;
+constexpr int kTopMaxK = 32;
+constexpr int kTopPerThread = 8;
+constexpr int kTopTile = kTopPerThread * kTopThreads;  // entries read together
+constexpr int kTopCap = 3584;                          // list entries (43 KB)
+constexpr int kTopSlots = kTopCap / kTopThreads;       // list entries a lane takes in a cut
+static_assert(kTopCap % kTopThreads == 0 && kTopCap >= kTopTile + kTopMaxK, "a cut list takes a whole tile");
 
-struct VI {
-  int64_t v;
-  int64_t i;
+struct TopShared {
+  int64_t v[kTopCap];
+  int32_t i[kTopCap];
+  int64_t wv[kTopWarps * kTopMaxK];  // each warp's k best
+  int32_t wi[kTopWarps * kTopMaxK];
+  int n;
 };
 
-__device__ __forceinline__ bool before(const VI& a, const VI& b) {  // a ranks ahead of b
-  return a.v > b.v || (a.v == b.v && a.i < b.i);
+// a ranks ahead of b
+__device__ __forceinline__ bool before(int64_t av, int32_t ai, int64_t bv, int32_t bi) {
+  return av > bv || (av == bv && ai < bi);
 }
 
-__device__ VI block_best(VI x, VI* sm) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// The k best of the entries base + stride q < m, q = 0..N-1, of lists V and I,
+// in order, to ov / oi (value 0 past the last positive one).  Whole warp.
+template <int N>
+__device__ __forceinline__ void warp_top(const int64_t* V, const int32_t* I, int m, int base, int stride, int k,
+                                         int64_t* ov, int32_t* oi, int lane) {
+  int64_t v[N];
+  int32_t id[N];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    VI y{__shfl_xor_sync(kFull, x.v, o), __shfl_xor_sync(kFull, x.i, o)};
-    if (before(y, x)) x = y;
+  for (int q = 0; q < N; ++q) {
+    const int at = base + stride * q;
+    v[q] = at < m ? V[at] : 0;
+    id[q] = at < m ? I[at] : INT32_MAX;
   }
-  if (lane == 0) sm[warp] = x;
-  __syncthreads();
-  VI r = sm[0];
-  for (int i = 1; i < kTopThreads / 32; ++i)
-    if (before(sm[i], r)) r = sm[i];
-  __syncthreads();
-  return r;
+  for (int r = 0; r < k; ++r) {
+    int64_t bv = 0;  // this lane's best
+    int32_t bi = INT32_MAX;
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (before(v[q], id[q], bv, bi)) {
+        bv = v[q];
+        bi = id[q];
+      }
+    const int64_t mv = static_cast<int64_t>(warp_max_u64(static_cast<uint64_t>(bv)));
+    const int32_t mi = __reduce_min_sync(kFull, bv == mv ? bi : INT32_MAX);
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (id[q] == mi) v[q] = 0, id[q] = INT32_MAX;  // indices are unique: only the pick goes
+    if (lane == 0) {
+      ov[r] = mv;
+      oi[r] = mi;
+    }
+  }
+  __syncwarp();
 }
 
-// A window's (stage, rank) entries are split over a cluster of kTopCluster
-// CTAs.  Each CTA finds the top k of its slice (k rounds of a block arg-max,
-// each round taking the best entry ranked after the previous pick), parks them
-// in its shared memory, and the cluster's first CTA merges the cluster's
-// k x kTopCluster candidates read through distributed shared memory.
-constexpr int kTopCluster = 8;
+// Cuts the CTA's list of m entries to its k best, in order.  Every thread calls it.
+__device__ __forceinline__ void cut_list(TopShared& sh, int m, int k) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int64_t* wv = sh.wv + warp * k;
+  int32_t* wi = sh.wi + warp * k;
+  if (m <= 4 * kTopThreads)
+    warp_top<4>(sh.v, sh.i, m, threadIdx.x, kTopThreads, k, wv, wi, lane);
+  else
+    warp_top<kTopSlots>(sh.v, sh.i, m, threadIdx.x, kTopThreads, k, wv, wi, lane);
+  __syncthreads();  // the list has been read, the warps' picks are written
+  if (warp == 0) {
+    warp_top<kTopMaxK * kTopWarps / 32>(sh.wv, sh.wi, kTopWarps * k, lane, 32, k, sh.v, sh.i, lane);
+    if (lane == 0) sh.n = k;
+  }
+  __syncthreads();
+}
 
-__global__ void __cluster_dims__(kTopCluster, 1, 1) __launch_bounds__(kTopThreads)
+__global__ void __launch_bounds__(kTopThreads)
     topk_kernel(const int64_t* __restrict__ X, const int64_t* __restrict__ E, int64_t S, int64_t R, int k,
                 int32_t* top_stage, int64_t* top_stage_value, int32_t* top_pair, int64_t* top_pair_value) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
-  __shared__ VI sm[kTopThreads / 32];
-  __shared__ VI cand[32];
-  const unsigned part = cluster.block_rank();
-  const int64_t w = blockIdx.x / kTopCluster;
+  __shared__ TopShared sh;
+  const int csize = static_cast<int>(cluster.num_blocks());
+  const int part = static_cast<int>(cluster.block_rank());
+  const int64_t w = blockIdx.x / csize;
+  const int lane = threadIdx.x & 31;
+  const bool pairs = E != nullptr && (top_pair != nullptr || top_pair_value != nullptr);  // uniform over the grid
+  const int n = static_cast<int>(S * R);  // <= 2^21
+  const int chunk = (n + csize - 1) / csize;
+  const int lo = min(part * chunk, n), hi = min(lo + chunk, n);
+  const int64_t* Ew = E + w * n;
+  int64_t next[kTopPerThread];
+  auto load_tile = [&](int at) {
+#pragma unroll
+    for (int q = 0; q < kTopPerThread; ++q) {
+      const int j = at + q * kTopThreads + static_cast<int>(threadIdx.x);
+      next[q] = j < hi ? __ldg(Ew + j) : 0;
+    }
+  };
+  if (pairs) load_tile(lo);
   if (part == 0 && threadIdx.x < 32 && (top_stage || top_stage_value)) {
-    const int lane = threadIdx.x;
     const int64_t v = lane < S ? X[w * S + lane] : 0;
     bool taken = false;
     for (int i = 0; i < k; ++i) {
@@ -497,41 +565,49 @@ __global__ void __cluster_dims__(kTopCluster, 1, 1) __launch_bounds__(kTopThread
       }
     }
   }
-  if (E == nullptr || (top_pair == nullptr && top_pair_value == nullptr)) return;  // uniform over the cluster
-  const int64_t n = S * R;
-  const int64_t chunk = (n + kTopCluster - 1) / kTopCluster;
-  const int64_t lo = part * chunk, hi = lo + chunk < n ? lo + chunk : n;
-  const int64_t* Ew = E + w * n;
-  VI prev{INT64_MAX, -1};
-  for (int i = 0; i < k; ++i) {
-    VI best{0, INT64_MAX};
-    if (prev.v > 0)
-      for (int64_t j = lo + threadIdx.x; j < hi; j += kTopThreads) {
-        const VI c{Ew[j], j};
-        if (c.v > 0 && before(prev, c) && before(c, best)) best = c;  // ranked after the last pick
+  if (!pairs) return;
+  if (threadIdx.x == 0) sh.n = 0;
+  __syncthreads();
+  for (int at = lo; at < hi; at += kTopTile) {
+    if (sh.n + kTopTile > kTopCap) cut_list(sh, sh.n, k);  // the same count in every thread
+    int64_t cur[kTopPerThread];
+#pragma unroll
+    for (int q = 0; q < kTopPerThread; ++q) cur[q] = next[q];
+    if (at + kTopTile < hi) load_tile(at + kTopTile);
+    __syncthreads();  // every thread has read the count
+#pragma unroll
+    for (int q = 0; q < kTopPerThread; ++q) {
+      const unsigned hit = __ballot_sync(kFull, cur[q] > 0);
+      if (hit == 0) continue;
+      int base = 0;
+      if (lane == 0) base = atomicAdd(&sh.n, __popc(hit));
+      base = __shfl_sync(kFull, base, 0) + __popc(hit & ((1u << lane) - 1u));
+      if (cur[q] > 0) {
+        sh.v[base] = cur[q];
+        sh.i[base] = at + q * kTopThreads + static_cast<int>(threadIdx.x);
       }
-    best = block_best(best, sm);
-    if (threadIdx.x == 0) cand[i] = best;
-    prev = best.v > 0 ? best : VI{0, INT64_MAX};
+    }
+    __syncthreads();
   }
+  cut_list(sh, sh.n, k);  // the list starts with the slice's k best
   cluster.sync();
-  if (part == 0) {
-    const int t = threadIdx.x;
-    VI mine{0, INT64_MAX};
-    if (t < kTopCluster * k) mine = cluster.map_shared_rank(cand, static_cast<unsigned>(t / k))[t % k];
-    prev = VI{INT64_MAX, -1};
-    for (int i = 0; i < k; ++i) {
-      VI c = (mine.v > 0 && before(prev, mine)) ? mine : VI{0, INT64_MAX};
-      c = block_best(c, sm);
-      if (threadIdx.x == 0) {
-        const bool ok = c.v > 0;
-        if (top_pair) {
-          top_pair[(w * k + i) * 2 + 0] = ok ? static_cast<int32_t>(c.i / R) : -1;
-          top_pair[(w * k + i) * 2 + 1] = ok ? static_cast<int32_t>(c.i % R) : -1;
-        }
-        if (top_pair_value) top_pair_value[w * k + i] = ok ? c.v : 0;
+  if (part == 0 && threadIdx.x < 32) {
+    // the candidates of all CTAs into this CTA's spare lists, then one cut
+    for (int c = lane; c < csize * k; c += 32) {
+      const unsigned from = static_cast<unsigned>(c / k);
+      sh.wv[c] = cluster.map_shared_rank(sh.v, from)[c % k];
+      sh.wi[c] = cluster.map_shared_rank(sh.i, from)[c % k];
+    }
+    __syncwarp();
+    warp_top<kTopMaxK * kTopCluster / 32>(sh.wv, sh.wi, csize * k, lane, 32, k, sh.v + kTopMaxK, sh.i + kTopMaxK, lane);
+    if (lane < k) {
+      const int64_t v = sh.v[kTopMaxK + lane];
+      const int32_t i = sh.i[kTopMaxK + lane];
+      if (top_pair) {
+        top_pair[(w * k + lane) * 2 + 0] = v > 0 ? static_cast<int32_t>(i / R) : -1;
+        top_pair[(w * k + lane) * 2 + 1] = v > 0 ? static_cast<int32_t>(i % R) : -1;
       }
-      prev = c.v > 0 ? c : VI{0, INT64_MAX};
+      if (top_pair_value) top_pair_value[w * k + lane] = v;
     }
   }
   cluster.sync();  // the other CTAs' candidates stay in place until the merge has read them
@@ -539,9 +615,14 @@ __global__ void __cluster_dims__(kTopCluster, 1, 1) __launch_bounds__(kTopThread
 
 // ---------------------------------------------------------------------------
 // Gates (App. C).  One CTA per window: the CTA scans rank roles and splits the
-// window's step leaders into 256 segments for the switch count; thread 0 then
-// evaluates the gates with exact integer comparisons a*den <op> num*b.
+// window's step leaders into 256 segments whose switch counts are joined in
+// order by warp shuffles; the first warp then evaluates the gates, lane s for
+// stage s, with exact integer comparisons a*den <op> num*b.  A few dependent
+// loads and shuffles are all there is to wait for: 4.3-5.0 us for 1 to 100
+// windows, where one thread that joined the segments and walked the stages
+// took 15-19 us.
 constexpr int kGateThreads = 256;
+constexpr int kGateWarps = kGateThreads / 32;
 
 __device__ __forceinline__ bool r_gt(__int128 lhs, sf_ratio r, __int128 rhs) {
   return lhs * r.den > static_cast<__int128>(r.num) * rhs;
@@ -553,54 +634,78 @@ __device__ __forceinline__ bool r_ge(__int128 lhs, sf_ratio r, __int128 rhs) {
   return lhs * r.den >= static_cast<__int128>(r.num) * rhs;
 }
 
-__global__ void __launch_bounds__(kGateThreads) gates_kernel(const GateJob g) {
-  __shared__ int seg_e[kGateThreads], seg_sw[kGateThreads], seg_first[kGateThreads],
-      seg_last[kGateThreads];
-  const int64_t w = blockIdx.x;
-  const int64_t S = g.S;
-  const int64_t tb = w * g.W, te = min(tb + g.W, g.T), n = te - tb;
-  int mixed = 0;
-  if (g.role) {
-    const int32_t r0 = g.role[0];
-    for (int64_t r = 1 + threadIdx.x; r < g.R; r += kGateThreads) mixed |= g.role[r] != r0;
+// The confident steps of a range: their count, the leader changes between
+// consecutive ones, the first and the last leader.
+struct LeadSeg {
+  int e = 0, sw = 0, first = -1, last = -1;
+  __device__ __forceinline__ void join(const LeadSeg& o) {  // o follows this range
+    if (o.e == 0) return;
+    sw += o.sw + (e != 0 && last != o.first ? 1 : 0);
+    if (e == 0) first = o.first;
+    last = o.last;
+    e += o.e;
   }
-  mixed = __syncthreads_or(mixed);
+};
+
+// Joins the segments of `n` (a power of two) consecutive lanes into the first one.
+__device__ __forceinline__ void join_lanes(LeadSeg& s, int n) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    if (o >= n) break;
+    LeadSeg up;
+    up.e = __shfl_down_sync(kFull, s.e, o);
+    up.sw = __shfl_down_sync(kFull, s.sw, o);
+    up.first = __shfl_down_sync(kFull, s.first, o);
+    up.last = __shfl_down_sync(kFull, s.last, o);
+    if ((threadIdx.x & (2 * o - 1)) == 0) s.join(up);
+  }
+}
+
+__global__ void __launch_bounds__(kGateThreads) gates_kernel(const GateJob g) {
+  __shared__ LeadSeg wseg[kGateWarps];
+  const int64_t w = blockIdx.x;
+  const int S = static_cast<int>(g.S);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool valid = lane < S;
+  const int64_t tb = w * g.W, te = min(tb + g.W, g.T), n = te - tb;
+  int64_t x = 0, y = 0, D = 0;
+  if (warp == 0) {
+    x = valid ? g.X[w * S + lane] : 0;
+    y = valid ? g.Y[w * S + lane] : 0;
+    D = g.D[w];
+  }
+  LeadSeg seg;
   {
     const int j = threadIdx.x;
     const int64_t sb = tb + n * j / kGateThreads, se = tb + n * (j + 1) / kGateThreads;
-    int e = 0, sw = 0, first = -1, last = -1;
+#pragma unroll 4
     for (int64_t t = sb; t < se; ++t) {
       const uint8_t sl = g.step_lead[t];
       if (sl & SF_STEP_CONFIDENT) {
         const int ld = sl & 31;
-        if (last >= 0 && ld != last) ++sw;
-        if (first < 0) first = ld;
-        last = ld;
-        ++e;
+        if (seg.e != 0 && ld != seg.last) ++seg.sw;
+        if (seg.e == 0) seg.first = ld;
+        seg.last = ld;
+        ++seg.e;
       }
     }
-    seg_e[j] = e;
-    seg_sw[j] = sw;
-    seg_first[j] = first;
-    seg_last[j] = last;
   }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-
-  int64_t e = 0, sw = 0;
-  int last = -1;
-  for (int j = 0; j < kGateThreads; ++j) {
-    if (seg_e[j] == 0) continue;
-    e += seg_e[j];
-    sw += seg_sw[j] + ((last >= 0 && seg_first[j] != last) ? 1 : 0);
-    last = seg_last[j];
+  int mixed = 0;
+  if (g.role) {
+    const int32_t r0 = g.role[0];
+#pragma unroll 8
+    for (int64_t r = 1 + threadIdx.x; r < g.R; r += kGateThreads) mixed |= g.role[r] != r0;
   }
+  join_lanes(seg, 32);
+  if (lane == 0) wseg[warp] = seg;
+  mixed = __syncthreads_or(mixed);
+  if (warp != 0) return;
+  seg = lane < kGateWarps ? wseg[lane] : LeadSeg();
+  join_lanes(seg, kGateWarps);
+  const int64_t e = __shfl_sync(kFull, seg.e, 0), sw = __shfl_sync(kFull, seg.sw, 0);
   const sf_label_config& c = g.cfg;
   const bool high_switch = e >= 2 && r_ge(e, c.gamma_elig, n) && r_gt(sw, c.gamma_switch, e - 1);
 
-  const int64_t* Xw = g.X + w * S;
-  const int64_t* Yw = g.Y + w * S;
-  const int64_t Dw = g.D[w];
   bool tel = g.missing != nullptr && g.missing[w] > c.max_missing_ranks;
   if (g.quality) {
     const uint64_t* q = g.quality + w * 6;
@@ -610,7 +715,7 @@ __global__ void __launch_bounds__(kGateThreads) gates_kernel(const GateJob g) {
     if (res * static_cast<uint64_t>(c.closure_max.den) > ws * static_cast<uint64_t>(c.closure_max.num)) tel = true;
     if (ovl * static_cast<uint64_t>(c.overlap_max.den) > ws * static_cast<uint64_t>(c.overlap_max.num)) tel = true;
   }
-  const bool raw = Dw < c.denom_floor_ns || Dw == 0;
+  const bool raw = D < c.denom_floor_ns || D == 0;
   if (raw) tel = true;
   uint32_t lab = SF_LABEL_FRONTIER_ACCOUNTING, route = 0, amb = 0;
   if (tel) lab |= SF_LABEL_TELEMETRY_LIMITED;
@@ -618,52 +723,50 @@ __global__ void __launch_bounds__(kGateThreads) gates_kernel(const GateJob g) {
   if (raw) {
     lab |= SF_LABEL_RAW_ONLY;
   } else {
-    int s1 = 0, g1 = 0;
-    for (int s = 1; s < S; ++s) {
-      if (Xw[s] > Xw[s1]) s1 = s;
-      if (Yw[s] > Yw[g1]) g1 = s;
-    }
-    int nA = 0, nG = 0;
-    for (int s = 0; s < S; ++s) {
-      if (r_lt(Xw[s1] - Xw[s], c.eta_A, Dw)) {
-        amb |= 1u << s;
-        ++nA;
+    // lowest stage with the largest X (Y): order-preserving unsigned keys
+    constexpr uint64_t kSign = 1ull << 63;
+    const uint64_t kx = static_cast<uint64_t>(x) ^ kSign, ky = static_cast<uint64_t>(y) ^ kSign;
+    const uint64_t mx = warp_max_u64(valid ? kx : 0ull), my = warp_max_u64(valid ? ky : 0ull);
+    const int s1 = __ffs(__ballot_sync(kFull, valid && kx == mx)) - 1;
+    const int64_t x1 = static_cast<int64_t>(mx ^ kSign), y1 = static_cast<int64_t>(my ^ kSign);
+    const uint32_t mA = __ballot_sync(kFull, valid && r_lt(x1 - x, c.eta_A, D));
+    const uint32_t mG = __ballot_sync(kFull, valid && r_lt(y1 - y, c.eta_G, D));
+    amb = mA | mG;
+    // leading-share prefix reaching tau_C: a stage is in it when no stage
+    // ranks ahead of it or the sum of those that do falls short
+    int64_t ahead = 0;
+    bool first = true;
+    for (int q = 0; q < S; ++q) {
+      const int64_t xq = __shfl_sync(kFull, x, q);
+      if (xq > x || (xq == x && q < lane)) {
+        ahead += xq;
+        first = false;
       }
-      if (r_lt(Yw[g1] - Yw[s], c.eta_G, Dw)) {
-        amb |= 1u << s;
-        ++nG;
-      }
     }
-    __int128 cum = 0;
-    for (int i = 0; i < S; ++i) {  // leading-share prefix reaching tau_C
-      int pick = -1;
-      for (int s = 0; s < S; ++s)
-        if (!((route >> s) & 1u) && (pick < 0 || Xw[s] > Xw[pick])) pick = s;
-      route |= 1u << pick;
-      cum += Xw[pick];
-      if (r_ge(cum, c.tau_C, Dw)) break;
-    }
-    const bool hiA = r_gt(Xw[s1], c.gamma_A, Dw);
-    const bool loG = r_lt(Yw[s1], c.gamma_G, Dw);
+    route = __ballot_sync(kFull, valid && (first || !r_ge(ahead, c.tau_C, D)));
+    const bool hiA = r_gt(x1, c.gamma_A, D);
+    const bool loG = r_lt(__shfl_sync(kFull, y, s1), c.gamma_G, D);
     const bool W1 = (c.model_fit_mask >> s1) & 1u;
-    const bool gain_tie = nG >= 2 && r_ge(Yw[g1], c.gamma_G, Dw);
+    const bool gain_tie = __popc(mG) >= 2 && r_ge(y1, c.gamma_G, D);
     if (hiA && loG) lab |= W1 ? SF_LABEL_SYNC_WAIT_DEPENDENT : SF_LABEL_CO_CRITICAL;
     if (hiA && !loG) lab |= SF_LABEL_DIRECT_EXPOSURE;
-    if (nA >= 2 || gain_tie || high_switch) {
+    if (__popc(mA) >= 2 || gain_tie || high_switch) {
       lab |= SF_LABEL_CO_CRITICAL;
       lab &= ~(SF_LABEL_DIRECT_EXPOSURE | SF_LABEL_SYNC_WAIT_DEPENDENT);
     }
     if (tel || mixed) lab &= ~(SF_LABEL_DIRECT_EXPOSURE | SF_LABEL_SYNC_WAIT_DEPENDENT);
   }
-  g.labels[w] = lab;
-  g.route_mask[w] = route;
-  g.amb_mask[w] = amb;
-  for (int s = 0; s < S; ++s) {
-    if (g.share) g.share[w * S + s] = raw ? 0.0 : static_cast<double>(Xw[s]) / static_cast<double>(Dw);
-    if (g.gain) g.gain[w * S + s] = raw ? 0.0 : static_cast<double>(Yw[s]) / static_cast<double>(Dw);
+  if (valid) {
+    if (g.share) g.share[w * S + lane] = raw ? 0.0 : static_cast<double>(x) / static_cast<double>(D);
+    if (g.gain) g.gain[w * S + lane] = raw ? 0.0 : static_cast<double>(y) / static_cast<double>(D);
   }
-  if (g.n_confident) g.n_confident[w] = static_cast<int32_t>(e);
-  if (g.n_switch) g.n_switch[w] = static_cast<int32_t>(sw);
+  if (lane == 0) {
+    g.labels[w] = lab;
+    g.route_mask[w] = route;
+    g.amb_mask[w] = amb;
+    if (g.n_confident) g.n_confident[w] = static_cast<int32_t>(e);
+    if (g.n_switch) g.n_switch[w] = static_cast<int32_t>(sw);
+  }
 }
 
 template <int NPL>
@@ -808,10 +911,27 @@ cudaError_t launch_window_median(const int64_t* d, int64_t T, int64_t R, int64_t
 cudaError_t launch_topk(const int64_t* X, const int64_t* E, int64_t nW, int64_t S, int64_t R, int32_t k,
                         int32_t* top_stage, int64_t* top_stage_value, int32_t* top_pair,
                         int64_t* top_pair_value, cudaStream_t stream) {
+  // one tile of entries per CTA, at most kTopCluster CTAs: more CTAs than that
+  // have nothing to read, and pay for their cut and the cluster's barriers
+  // (100 windows of 128 x 8 entries, k = 2: 15.4 us with clusters of eight, 6.4 us
+  // with one CTA each)
+  const int64_t n = E && (top_pair || top_pair_value) ? S * R : 1;
+  unsigned csize = 1;
+  while (csize < kTopCluster && int64_t(csize) * kTopTile < n) csize *= 2;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = csize;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(nW * csize));
+  cfg.blockDim = dim3(kTopThreads);
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
   count_launch();
-  topk_kernel<<<static_cast<unsigned>(nW * kTopCluster), kTopThreads, 0, stream>>>(
-      X, E, S, R, k, top_stage, top_stage_value, top_pair, top_pair_value);
-  return cudaGetLastError();
+  return cudaLaunchKernelEx(&cfg, topk_kernel, X, E, S, R, static_cast<int>(k), top_stage, top_stage_value, top_pair,
+                            top_pair_value);
 }
 
 cudaError_t launch_gates(const GateJob& job, cudaStream_t stream) {

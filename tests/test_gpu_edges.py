@@ -1,0 +1,63 @@
+"""GPU parity at the sizes where one kernel form gives way to another: tile
+and list edges, remainders, and the smallest and largest of a form's range.
+Every output is compared with the CPU oracle, whole numbers exactly."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sf():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2606_06751_gb300 import build as B
+    B.build()
+    from paper_2606_06751_gb300 import stagefrontier
+    return stagefrontier
+
+
+def dev(x):
+    return torch.from_numpy(np.ascontiguousarray(x)).cuda()
+
+
+def host(t):
+    return t.cpu().numpy()
+
+
+# one tile of entries and one more, cluster sizes 1 to 8, lists that overflow
+# (every entry positive) and sparse ones, ties across CTAs, k of 1 and 32
+@pytest.mark.parametrize("nW,S,R,k", [(3, 1, 2048, 5), (2, 1, 2049, 32), (2, 2, 2049, 32), (1, 3, 5461, 7),
+                                      (2, 8, 2049, 32), (1, 8, 8192, 32), (1, 5, 16385, 1)])
+@pytest.mark.parametrize("positive", [1.0, 0.05, 0.0])
+def test_topk_lists(sf, nW, S, R, k, positive):
+    rng = np.random.default_rng(S * R + k)
+    X = rng.integers(0, 4, size=(nW, S)).astype(np.int64)
+    E = rng.integers(1, 50, size=(nW, S, R)).astype(np.int64) << 40
+    E[rng.random(E.shape) >= positive] = 0
+    o = O.topk(X, E, k)
+    t = sf.sf_topk_suspects(dev(X), dev(E), k)
+    assert np.array_equal(host(t.stage), o.stage) and np.array_equal(host(t.stage_value), o.stage_value)
+    assert np.array_equal(host(t.pair), o.pair) and np.array_equal(host(t.pair_value), o.pair_value)
+
+
+# windows shorter and longer than the gate kernel's 256 segments, up to 32
+# stages, leaders that change within and across segments and unsure steps
+@pytest.mark.parametrize("T,S,W", [(30, 2, 7), (600, 5, 255), (1025, 31, 512), (3000, 32, 3000), (700, 1, 256)])
+def test_gates_switches(sf, T, S, W):
+    rng = np.random.default_rng(T + S)
+    d = rng.integers(1, 1000, size=(T, 2, S)).astype(np.int64)
+    runs = np.repeat(rng.integers(0, S, size=T), rng.integers(1, 6, size=T))[:T]
+    lead = rng.random(T) < 0.8
+    d[np.nonzero(lead)[0], :, runs[lead]] += 50000
+    o = O.label_windows(d, W)
+    m = sf.sf_window_median(dev(d), W)
+    ev = sf.sf_direct_gain(dev(d), W, m)
+    g = sf.sf_label_gates(T, 2, S, W, ev)
+    assert np.array_equal(host(g.n_confident), o.n_confident) and np.array_equal(host(g.n_switch), o.n_switch)
+    for got, want in ((g.labels, o.labels), (g.route_mask, o.route_mask), (g.amb_mask, o.amb_mask)):
+        assert np.array_equal(host(got).astype(np.uint32), want)
+    assert np.array_equal(host(g.share), o.share) and np.array_equal(host(g.gain), o.gain)
