@@ -4,14 +4,24 @@
 // the frontier.  1 means the lead rank is the unique one; more means a tie
 // that the frontier pass resolved to the lowest rank.
 //
-// One more pass over d: one CTA per step range; per step, the frontier
-// F[t,s] is rebuilt from the increments a[t,.] of the frontier pass (their
-// prefix over s), every thread counts, per stage, its rank rows whose prefix
-// equals it, and the counts are summed over the CTA.  The per-stage state is
-// sized by a bound SMAX >= S with every stage loop unrolled to SMAX behind an
-// `s < S` test, so it stays in registers.
+// One more pass over d: per step, the frontier F[t,s] is rebuilt from the
+// increments a[t,.] of the frontier pass (their prefix over s), every thread
+// counts, per stage, its rank rows whose prefix equals it, and the counts are
+// summed.  Three splits of the work, chosen by launch_frontier_ties:
+//   ties_warp_kernel - up to kTieWarpRanks ranks and enough steps to fill the
+//     chip with warps: a warp per step, no CTA barrier.  Three barriers a step
+//     bound small steps (100000 x 128 x 8: 344 us with a CTA per step, 136 us,
+//     90 % of the measured copy rate, with a warp);
+//   ties_kernel      - a CTA per step, the CTA walking a range of steps; with
+//     fewer steps than the chip holds CTAs, a thread-block cluster per step,
+//     its CTAs' counts summed through distributed shared memory (one step of
+//     8192 x 8: 19.8 us in one CTA, 8.3 us in a cluster of eight).
+// The per-stage state is sized by a bound SMAX >= S with every stage loop
+// unrolled to SMAX behind an `s < S` test, so it stays in registers.
 #include <algorithm>
 #include <type_traits>
+
+#include <cooperative_groups.h>
 
 #include "sf_device.cuh"
 #include "sf_launch.h"
@@ -22,30 +32,109 @@ namespace {
 
 constexpr int kTieThreads = 256;
 constexpr int kTieWarps = kTieThreads / 32;
+constexpr int64_t kTieWarpRanks = 512;
+constexpr int kTieCluster = 8;
 
 __device__ __forceinline__ uint32_t hi32(int64_t v) {
   return static_cast<uint32_t>(static_cast<uint64_t>(v) >> 32);
 }
 
+// Lane s < S: F[t,s], the inclusive prefix of the increments over s.
+__device__ __forceinline__ int64_t lane_frontier(const int64_t* a, int64_t t, int S, int lane) {
+  int64_t x = lane < S ? __ldg(a + t * S + lane) : 0;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t up = __shfl_up_sync(kFull, x, o);
+    if (lane >= o) x += up;
+  }
+  return x;
+}
+
+// Counts the rows r0, r0 + stride, ... < r1 of a step whose prefix equals F.
 // VEC: S even, rows start 16-byte aligned and are read with 16-byte loads.
 template <int SMAX, bool VEC>
+__device__ __forceinline__ void count_rows(const int64_t* dt, int S, int r0, int r1, int stride,
+                                           const int64_t (&F)[SMAX], uint32_t (&cnt)[SMAX], uint32_t& dor,
+                                           uint32_t& tor) {
+  for (int r = r0; r < r1; r += stride) {
+    const int64_t* row = dt + int64_t(r) * S;
+    int64_t P = 0;
+    if constexpr (VEC) {
+#pragma unroll
+      for (int s = 0; s < SMAX; s += 2) {
+        if (s >= S) break;
+        const longlong2 x = __ldg(reinterpret_cast<const longlong2*>(row + s));
+        dor |= hi32(x.x) | hi32(x.y);
+        P += x.x;
+        cnt[s] += P == F[s] ? 1u : 0u;
+        P += x.y;
+        cnt[s + 1] += P == F[s + 1] ? 1u : 0u;
+      }
+    } else {
+#pragma unroll
+      for (int s = 0; s < SMAX; ++s) {
+        if (s >= S) break;
+        const int64_t v = __ldg(row + s);
+        dor |= hi32(v);
+        P += v;
+        cnt[s] += P == F[s] ? 1u : 0u;
+      }
+    }
+    tor |= hi32(P);
+  }
+}
+
+template <int SMAX, bool VEC>
 __global__ void __launch_bounds__(kTieThreads)
-    ties_kernel(const int64_t* __restrict__ d, int64_t T, int64_t R, int S, const int64_t* __restrict__ a,
+    ties_warp_kernel(const int64_t* __restrict__ d, int64_t T, int R, int S, const int64_t* __restrict__ a,
+                     int32_t* __restrict__ ties, uint32_t* status) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = int64_t(gridDim.x) * kTieWarps, id = int64_t(blockIdx.x) * kTieWarps + (threadIdx.x >> 5);
+  uint32_t dor = 0, tor = 0;
+  for (int64_t t = id; t < T; t += nw) {
+    const int64_t x = lane_frontier(a, t, S, lane);
+    int64_t F[SMAX];
+    uint32_t cnt[SMAX];
+#pragma unroll
+    for (int s = 0; s < SMAX; ++s) {
+      if (s >= S) break;
+      F[s] = __shfl_sync(kFull, x, s);
+      cnt[s] = 0;
+    }
+    count_rows<SMAX, VEC>(d + t * R * S, S, lane, R, 32, F, cnt, dor, tor);
+    uint32_t mine = 0;
+#pragma unroll
+    for (int s = 0; s < SMAX; ++s) {
+      if (s >= S) break;
+      const uint32_t c = __reduce_add_sync(kFull, cnt[s]);
+      if (lane == s) mine = c;
+    }
+    if (lane < S) ties[t * S + lane] = static_cast<int32_t>(mine);
+  }
+  const uint32_t bits = range_bits(__reduce_or_sync(kFull, dor), __reduce_or_sync(kFull, tor));
+  if (lane == 0) report(status, bits);
+}
+
+// A cluster of CTAs per step (of one CTA in most launches), each counting an
+// equal share of the ranks.
+template <int SMAX, bool VEC>
+__global__ void __launch_bounds__(kTieThreads)
+    ties_kernel(const int64_t* __restrict__ d, int64_t T, int R, int S, const int64_t* __restrict__ a,
                 int32_t* __restrict__ ties, uint32_t* status) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
   __shared__ int64_t sF[32];
   __shared__ uint32_t wcnt[kTieWarps][32];
+  __shared__ uint32_t sum[32];
+  const int csize = static_cast<int>(cluster.num_blocks()), part = static_cast<int>(cluster.block_rank());
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t NB = gridDim.x, b = blockIdx.x;
+  const int64_t NB = gridDim.x / csize, b = blockIdx.x / csize;
   const int64_t t_begin = T * b / NB, t_end = T * (b + 1) / NB;
+  const int r0 = static_cast<int>(int64_t(R) * part / csize), r1 = static_cast<int>(int64_t(R) * (part + 1) / csize);
   uint32_t dor = 0, tor = 0;
   for (int64_t t = t_begin; t < t_end; ++t) {
-    if (warp == 0) {  // F[t,s]: inclusive prefix of the increments over s
-      int64_t x = lane < S ? __ldg(a + t * S + lane) : 0;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int64_t up = __shfl_up_sync(kFull, x, o);
-        if (lane >= o) x += up;
-      }
+    if (warp == 0) {
+      const int64_t x = lane_frontier(a, t, S, lane);
       if (lane < S) sF[lane] = x;
     }
     __syncthreads();
@@ -57,32 +146,7 @@ __global__ void __launch_bounds__(kTieThreads)
       F[s] = sF[s];
       cnt[s] = 0;
     }
-    for (int64_t r = threadIdx.x; r < R; r += kTieThreads) {
-      const int64_t* row = d + (t * R + r) * S;
-      int64_t P = 0;
-      if constexpr (VEC) {
-#pragma unroll
-        for (int s = 0; s < SMAX; s += 2) {
-          if (s >= S) break;
-          const longlong2 x = __ldg(reinterpret_cast<const longlong2*>(row + s));
-          dor |= hi32(x.x) | hi32(x.y);
-          P += x.x;
-          cnt[s] += P == F[s] ? 1u : 0u;
-          P += x.y;
-          cnt[s + 1] += P == F[s + 1] ? 1u : 0u;
-        }
-      } else {
-#pragma unroll
-        for (int s = 0; s < SMAX; ++s) {
-          if (s >= S) break;
-          const int64_t v = __ldg(row + s);
-          dor |= hi32(v);
-          P += v;
-          cnt[s] += P == F[s] ? 1u : 0u;
-        }
-      }
-      tor |= hi32(P);
-    }
+    count_rows<SMAX, VEC>(d + t * R * S, S, r0 + static_cast<int>(threadIdx.x), r1, kTieThreads, F, cnt, dor, tor);
 #pragma unroll
     for (int s = 0; s < SMAX; ++s) {
       if (s >= S) break;
@@ -90,12 +154,19 @@ __global__ void __launch_bounds__(kTieThreads)
       if (lane == 0) wcnt[warp][s] = c;
     }
     __syncthreads();
+    uint32_t c = 0;
     if (warp == 0 && lane < S) {
-      uint32_t c = 0;
 #pragma unroll
       for (int w = 0; w < kTieWarps; ++w) c += wcnt[w][lane];
-      ties[t * S + lane] = static_cast<int32_t>(c);
+      sum[lane] = c;
     }
+    if (csize > 1) {
+      cluster.sync();  // every CTA's counts are written
+      if (part == 0 && warp == 0 && lane < S)
+        for (int q = 1; q < csize; ++q) c += *cluster.map_shared_rank(&sum[lane], static_cast<unsigned>(q));
+      cluster.sync();  // ... and read, before a CTA leaves or writes its next step's
+    }
+    if (part == 0 && warp == 0 && lane < S) ties[t * S + lane] = static_cast<int32_t>(c);
     __syncthreads();  // sF and wcnt are rewritten for the next step
   }
   const uint32_t bits = range_bits(__reduce_or_sync(kFull, dor), __reduce_or_sync(kFull, tor));
@@ -106,20 +177,40 @@ __global__ void __launch_bounds__(kTieThreads)
 
 cudaError_t launch_frontier_ties(const int64_t* d, int64_t T, int64_t R, int64_t S, const int64_t* a,
                                  int32_t* ties, uint32_t* status, cudaStream_t stream) {
-  const int grid = static_cast<int>(std::min<int64_t>(int64_t(sm_count()) * 4, T));
-  const bool vec = S % 2 == 0;
-  const int s = static_cast<int>(S);
-  auto go = [&](auto smax) {
+  const int s = static_cast<int>(S), r = static_cast<int>(R);
+  count_launch();
+  auto go = [&](auto smax, auto vec) {
     constexpr int SM = decltype(smax)::value;
-    count_launch();
-    if (vec) ties_kernel<SM, true><<<grid, kTieThreads, 0, stream>>>(d, T, R, s, a, ties, status);
-    else ties_kernel<SM, false><<<grid, kTieThreads, 0, stream>>>(d, T, R, s, a, ties, status);
-    return cudaGetLastError();
+    constexpr bool V = decltype(vec)::value;
+    const int64_t ctas = int64_t(sm_count()) * 4;
+    if (R <= kTieWarpRanks && (T >= ctas || R <= 64)) {
+      const int grid = static_cast<int>(std::min<int64_t>(2 * ctas, (T + kTieWarps - 1) / kTieWarps));
+      ties_warp_kernel<SM, V><<<grid, kTieThreads, 0, stream>>>(d, T, r, s, a, ties, status);
+      return cudaGetLastError();
+    }
+    // few steps: CTAs of a cluster share one, each with at least two rows a thread
+    unsigned csize = 1;
+    while (csize < kTieCluster && T * csize * 2 <= ctas && R >= int64_t(csize) * 4 * kTieThreads) csize *= 2;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = csize;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(std::min<int64_t>(ctas / csize, T) * csize));
+    cfg.blockDim = dim3(kTieThreads);
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, ties_kernel<SM, V>, d, T, r, s, a, ties, status);
   };
-  if (S <= 4) return go(std::integral_constant<int, 4>{});
-  if (S <= 8) return go(std::integral_constant<int, 8>{});
-  if (S <= 16) return go(std::integral_constant<int, 16>{});
-  return go(std::integral_constant<int, 32>{});
+  auto pick = [&](auto smax) {
+    return S % 2 == 0 ? go(smax, std::true_type{}) : go(smax, std::false_type{});
+  };
+  if (S <= 4) return pick(std::integral_constant<int, 4>{});
+  if (S <= 8) return pick(std::integral_constant<int, 8>{});
+  if (S <= 16) return pick(std::integral_constant<int, 16>{});
+  return pick(std::integral_constant<int, 32>{});
 }
 
 }  // namespace sf

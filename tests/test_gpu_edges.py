@@ -61,3 +61,11 @@ def test_gates_switches(sf, T, S, W):
     for got, want in ((g.labels, o.labels), (g.route_mask, o.route_mask), (g.amb_mask, o.amb_mask)):
         assert np.array_equal(host(got).astype(np.uint32), want)
     assert np.array_equal(host(g.share), o.share) and np.array_equal(host(g.gain), o.gain)
+
+
+# a warp per step and a CTA or a cluster of CTAs per step
+@pytest.mark.parametrize("T,R,S", [(700, 512, 3), (700, 513, 8), (5, 64, 6), (1, 65, 16), (2, 2047, 5), (1, 8192, 8),
+                                   (16, 8191, 4), (300, 4096, 2), (1, 65536, 3), (2500, 40, 20)])
+def test_ties_splits(sf, T, R, S):
+    d_np = np.random.default_rng(T + R).integers(0, 4, size=(T, R, S)).astype(np.int64)
+    assert np.array_equal(host(sf.sf_frontier_ties(dev(d_np))), O.frontier(d_np).ties)
