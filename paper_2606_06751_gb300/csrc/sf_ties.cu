@@ -34,6 +34,8 @@ constexpr int kTieThreads = 256;
 constexpr int kTieWarps = kTieThreads / 32;
 constexpr int64_t kTieWarpRanks = 512;
 constexpr int kTieCluster = 8;
+// ties_kernel CTAs per SM
+constexpr int tie_ctas(int smax) { return smax == 16 ? 2 : 4; }
 
 __device__ __forceinline__ uint32_t hi32(int64_t v) {
   return static_cast<uint32_t>(static_cast<uint64_t>(v) >> 32);
@@ -51,33 +53,39 @@ __device__ __forceinline__ int64_t lane_frontier(const int64_t* a, int64_t t, in
 }
 
 // Counts the rows r0, r0 + stride, ... < r1 of a step whose prefix equals F.
-// VEC: S even, rows start 16-byte aligned and are read with 16-byte loads.
+// VEC: S even, rows start 16-byte aligned and are read with 16-byte loads.  With
+// 9 to 16 stages a row's loads are all issued before its first use (50000 x 1024 x
+// 10: 1100 -> 846 us); shorter rows gain nothing by it, longer ones cost too many
+// registers (1000 x 24: 141 against 189 us).
 template <int SMAX, bool VEC>
 __device__ __forceinline__ void count_rows(const int64_t* dt, int S, int r0, int r1, int stride,
                                            const int64_t (&F)[SMAX], uint32_t (&cnt)[SMAX], uint32_t& dor,
                                            uint32_t& tor) {
+  constexpr int kStage = SMAX == 16 ? SMAX : VEC ? 2 : 1;  // stages loaded together
   for (int r = r0; r < r1; r += stride) {
     const int64_t* row = dt + int64_t(r) * S;
     int64_t P = 0;
-    if constexpr (VEC) {
 #pragma unroll
-      for (int s = 0; s < SMAX; s += 2) {
-        if (s >= S) break;
-        const longlong2 x = __ldg(reinterpret_cast<const longlong2*>(row + s));
-        dor |= hi32(x.x) | hi32(x.y);
-        P += x.x;
-        cnt[s] += P == F[s] ? 1u : 0u;
-        P += x.y;
-        cnt[s + 1] += P == F[s + 1] ? 1u : 0u;
+    for (int s0 = 0; s0 < SMAX; s0 += kStage) {
+      if (s0 >= S) break;
+      int64_t v[kStage];
+#pragma unroll
+      for (int i = 0; i < kStage; i += VEC ? 2 : 1) {
+        if (s0 + i >= S) break;
+        if constexpr (VEC) {
+          const longlong2 x = __ldg(reinterpret_cast<const longlong2*>(row + s0 + i));
+          v[i] = x.x;
+          v[i + 1] = x.y;
+        } else {
+          v[i] = __ldg(row + s0 + i);
+        }
       }
-    } else {
 #pragma unroll
-      for (int s = 0; s < SMAX; ++s) {
-        if (s >= S) break;
-        const int64_t v = __ldg(row + s);
-        dor |= hi32(v);
-        P += v;
-        cnt[s] += P == F[s] ? 1u : 0u;
+      for (int i = 0; i < kStage; ++i) {
+        if (s0 + i >= S) break;
+        dor |= hi32(v[i]);
+        P += v[i];
+        cnt[s0 + i] += P == F[s0 + i] ? 1u : 0u;
       }
     }
     tor |= hi32(P);
@@ -118,7 +126,7 @@ __global__ void __launch_bounds__(kTieThreads)
 // A cluster of CTAs per step (of one CTA in most launches), each counting an
 // equal share of the ranks.
 template <int SMAX, bool VEC>
-__global__ void __launch_bounds__(kTieThreads)
+__global__ void __launch_bounds__(kTieThreads, SMAX <= 8 ? 4 : 2)
     ties_kernel(const int64_t* __restrict__ d, int64_t T, int R, int S, const int64_t* __restrict__ a,
                 int32_t* __restrict__ ties, uint32_t* status) {
   namespace cg = cooperative_groups;
@@ -182,9 +190,9 @@ cudaError_t launch_frontier_ties(const int64_t* d, int64_t T, int64_t R, int64_t
   auto go = [&](auto smax, auto vec) {
     constexpr int SM = decltype(smax)::value;
     constexpr bool V = decltype(vec)::value;
-    const int64_t ctas = int64_t(sm_count()) * 4;
+    const int64_t ctas = int64_t(sm_count()) * tie_ctas(SM);
     if (R <= kTieWarpRanks && (T >= ctas || R <= 64)) {
-      const int grid = static_cast<int>(std::min<int64_t>(2 * ctas, (T + kTieWarps - 1) / kTieWarps));
+      const int grid = static_cast<int>(std::min<int64_t>(int64_t(sm_count()) * 8, (T + kTieWarps - 1) / kTieWarps));
       ties_warp_kernel<SM, V><<<grid, kTieThreads, 0, stream>>>(d, T, r, s, a, ties, status);
       return cudaGetLastError();
     }
