@@ -10,6 +10,8 @@
 
 #include "sf_device.cuh"
 #include "sf_launch.h"
+#include "sf_lane_select.cuh"
+#include "sf_warp_select.cuh"
 
 namespace sf {
 
@@ -49,12 +51,6 @@ __global__ void zero_many_kernel(const ZeroList z) {
 // and the rank re-based into that bin.  A 24-bit spread takes three passes.
 constexpr int kMedCols = 8;
 constexpr int kMedThreads = kMedCols * 32;
-constexpr int kMedBins = 256;
-// Per-warp counters: 256 digit bins, then 48 spare words (a compacted bin of
-// at most 32 values and its padding to whole 16-byte groups).  304 words =
-// 1216 bytes keeps every warp's block 16-byte aligned.
-constexpr int kMedHistWords = kMedBins + 48;
-
 // k-th smallest (0-based) of the lane-strided values get(i) (row lane + 32 i,
 // valid while row < n), all below 2^nbits.  hist: this warp's 256 counters.
 template <typename U, int NPL, typename Get>
@@ -117,15 +113,6 @@ __device__ __forceinline__ U warp_radix_select(Get get, int n, int nbits, uint32
   return prefix;
 }
 
-// Shared-memory increment of one counter, issued only when `pred` is set
-// (explicitly predicated, so a warp never branches around it).
-__device__ __forceinline__ void red_shared_inc_if(uint32_t* counter, bool pred) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p red.shared.add.u32 [%0], 1;\n\t}" ::"r"(smem_u32(counter)),
-      "r"(static_cast<uint32_t>(pred))
-      : "memory");
-}
-
 template <int NPL, bool kVec>
 __global__ void __launch_bounds__(kMedThreads)
     median_kernel(const int64_t* __restrict__ d, int64_t T, int64_t RS, int64_t W, int64_t ngroups,
@@ -156,7 +143,7 @@ __global__ void __launch_bounds__(kMedThreads)
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp >= ncols) return;
-  uint32_t* hist = hists + warp * kMedBins;  // 1 KB per warp
+  uint32_t* hist = hists + warp * kSelBins;  // 1 KB per warp
   constexpr uint64_t kSign = 1ull << 63;
   uint64_t u[NPL];
   uint64_t lo = ~0ull, hi = 0;
@@ -186,79 +173,6 @@ __global__ void __launch_bounds__(kMedThreads)
     ans = warp_radix_select<uint64_t, NPL>([&](int i) { return u[i]; }, n, nbits, k, hist, lane);
   }
   if (lane == 0) m[w * RS + c0 + warp] = static_cast<int64_t>((lo + ans) ^ kSign);
-}
-
-// Radix selection on a column held in registers (x[i] = row lane + 32 i):
-// the k-th smallest of the live values, all below 2^nbits.  Padding slots
-// must hold 2^nbits - 1: they sort at or after every live value, so counting
-// them never moves the rank-k bin and no slot needs a validity test.  The
-// first digit is the top 8 bits of the range, [nbits - 8, nbits), so it
-// spreads over the 256 bins and its chosen bin usually holds a few percent of
-// the column; each later pass counts, predicated, the values that share the
-// digits chosen so far.  As soon as the chosen bin holds at most 32 values
-// they are compacted into the spare words after the bins (ballot ranks, no
-// atomics) and each is ranked by counting.
-template <int NPL>
-__device__ __forceinline__ uint32_t warp_select_regs(const uint32_t (&x)[NPL], int nbits, uint32_t k,
-                                                     uint32_t* hist, int lane) {
-  uint32_t prefix = 0, rem = k;
-  int hi = nbits;
-  bool first = true;
-  while (hi > 0) {
-    const int sh = hi > 8 ? hi - 8 : 0;
-    const uint32_t mask = (1u << (hi - sh)) - 1u;
-    reinterpret_cast<uint4*>(hist)[2 * lane] = make_uint4(0, 0, 0, 0);
-    reinterpret_cast<uint4*>(hist)[2 * lane + 1] = make_uint4(0, 0, 0, 0);
-    __syncwarp();
-    if (first) {
-#pragma unroll
-      for (int i = 0; i < NPL; ++i) atomicAdd(&hist[x[i] >> sh], 1u);  // x < 2^nbits: the bin is below 256
-    } else {
-#pragma unroll
-      for (int i = 0; i < NPL; ++i)
-        red_shared_inc_if(&hist[(x[i] >> sh) & mask], (x[i] >> hi) == (prefix >> hi));
-    }
-    __syncwarp();
-    uint32_t digit, below;
-    hist_find(hist, rem, lane, digit, below);
-    const uint32_t kept = hist[digit];
-    rem -= below;
-    prefix |= digit << sh;
-    hi = sh;
-    first = false;
-    if (hi > 0 && kept <= 32) {
-      uint32_t* cbuf = hist + kMedBins;
-      const uint32_t below_lane = (1u << lane) - 1u;
-      uint32_t base = 0;
-#pragma unroll
-      for (int i = 0; i < NPL; ++i) {
-        const bool mt = (x[i] >> hi) == (prefix >> hi);
-        const uint32_t mm = __ballot_sync(kFull, mt);
-        if (mm) {
-          if (mt) cbuf[base + __popc(mm & below_lane)] = x[i];
-          base += __popc(mm);
-        }
-      }
-      if (lane < 3) cbuf[kept + lane] = 0xffffffffu;  // pad to whole 16-byte groups (kept + 3 <= 35 < 64 spare)
-      __syncwarp();
-      // rank each bin value by counting (broadcast reads of the bin): the
-      // answer is a value with lt <= rem < le.  Padding counts only toward
-      // le of the largest key, which no rank below kept can need.
-      const uint32_t v = cbuf[lane & 31];
-      uint32_t lt = 0, le = 0;
-      for (uint32_t q = 0; q < kept; q += 4) {
-        const uint4 c = *reinterpret_cast<const uint4*>(cbuf + q);
-        lt += (c.x < v) + (c.y < v) + (c.z < v) + (c.w < v);
-        le += (c.x <= v) + (c.y <= v) + (c.z <= v) + (c.w <= v);
-      }
-      const uint32_t hit = __ballot_sync(kFull, static_cast<uint32_t>(lane) < kept && lt <= rem && rem < le);
-      const uint32_t ans = __shfl_sync(kFull, v, __ffs(hit) - 1);
-      __syncwarp();
-      return ans;
-    }
-    __syncwarp();
-  }
-  return prefix;
 }
 
 // Lower median of one column of n <= 32 NPL rows read from global memory
@@ -297,8 +211,14 @@ __device__ __noinline__ int64_t median_column_global(const int64_t* __restrict__
 // The selection touches only registers and the warp's counters.  A column
 // whose values do not share their high 32 bits selects on 64-bit values
 // re-read from d.  Every window of a launch holds the same n rows.
+//
+// Resident CTAs hide each tile's copy and selection chain, so the registers are
+// held to what the most CTAs allow without spilling the column (512-row columns,
+// 1024 x 10: three CTAs 832 us, four 824 us).
+constexpr int med_min_ctas(int npl) { return npl >= 32 ? 3 : npl == 16 ? 4 : 5; }
+
 template <int NPL, bool kFit>
-__global__ void __launch_bounds__(kMedThreads, 3)
+__global__ void __launch_bounds__(kMedThreads, med_min_ctas(NPL))
     median_persist_kernel(const __grid_constant__ CUtensorMap map, const int64_t* __restrict__ d, int64_t T,
                           int64_t RS, int64_t W, int64_t w0, int64_t nW, int64_t ngroups, int box_rows, int nbox,
                           int64_t* __restrict__ m, uint32_t* status) {
@@ -307,11 +227,11 @@ __global__ void __launch_bounds__(kMedThreads, 3)
   const uint32_t tile_bytes = uint32_t(nbox) * uint32_t(box_rows) * 64u;  // bytes the copies write
   const int tile_rows = max(nbox * box_rows, 32 * NPL);
   uint32_t* hists = reinterpret_cast<uint32_t*>(tile + uint32_t(tile_rows) * 64u);
-  uint64_t* full = reinterpret_cast<uint64_t*>(hists + kMedCols * kMedHistWords);
+  uint64_t* full = reinterpret_cast<uint64_t*>(hists + kMedCols * kSelHistWords);
   uint64_t* empty = full + 1;
   volatile int* abort = reinterpret_cast<volatile int*>(full + 2);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint32_t* hist = hists + warp * kMedHistWords;
+  uint32_t* hist = hists + warp * kSelHistWords;
   const int64_t ntiles = nW * ngroups;
   auto issue = [&](int64_t id) {  // one thread: the bulk copies of tile `id`
     const int64_t c0 = (id % ngroups) * kMedCols;
@@ -397,6 +317,77 @@ __global__ void __launch_bounds__(kMedThreads, 3)
       if (lane == 0) m[w * RS + c0 + warp] = med;
     }
   }
+}
+
+// Short windows (n <= 128 rows): one lane per column.  A warp takes 32
+// consecutive columns of a window, so its loads are whole 256-byte runs of d at
+// any alignment, and every lane holds its column in registers (32-bit keys, the
+// values' low words) and searches its own median without a word to the others
+// (lane_select).  A column whose values do not share their high words is taken
+// by the whole warp on 64-bit values.  Against a warp per column, whose histogram
+// and searches cost as much for a hundred rows as for a thousand: 100000 x 128 x 6
+// in windows of 100 steps 337 -> 188 us, one window of 100 x 8192 x 8 33 -> 22.5 us.
+// Bound by the loads a warp can hold beside its keys.
+constexpr int kLaneMedThreads = 128;
+constexpr int kLaneMedMaxRows = 128;
+
+template <int NMAX>
+__global__ void __launch_bounds__(kLaneMedThreads, lane_ctas(NMAX))
+    median_lanes_kernel(const int64_t* __restrict__ d, int64_t T, int64_t RS, int64_t W, int64_t tiles,
+                        int64_t ntiles, int64_t* __restrict__ m) {
+  constexpr int kBatch = lane_batch(NMAX);  // rows loaded together
+  __shared__ __align__(16) uint32_t hists[kLaneMedThreads / 32][kSelHistWords];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t nw = int64_t(gridDim.x) * (kLaneMedThreads / 32);
+  for (int64_t id = int64_t(blockIdx.x) * (kLaneMedThreads / 32) + warp; id < ntiles; id += nw) {
+    const int64_t w = id / tiles, c0 = (id - w * tiles) * 32, tb = w * W;
+    const int n = static_cast<int>(imin64(W, T - tb));
+    const bool mine = c0 + lane < RS;
+    const int64_t* col = d + tb * RS + c0 + (mine ? lane : 0);
+    uint32_t x[NMAX];
+    uint32_t hand = 0xffffffffu, hor = 0u;
+#pragma unroll
+    for (int b = 0; b < NMAX; b += kBatch) {
+      uint2 v[kBatch];
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) v[i] = load_words(col + min(b + i, n - 1) * RS);  // past the window: its last row
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        x[b + i] = b + i < n ? v[i].x : 0xffffffffu;  // sorts last
+        hand &= v[i].y;
+        hor |= v[i].y;
+      }
+    }
+    const uint32_t kth = static_cast<uint32_t>((n - 1) / 2);
+    uint32_t lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+    for (int i = 0; i < NMAX; ++i) {
+      lo = min(lo, x[i]);
+      hi = max(hi, i < n ? x[i] : 0u);
+    }
+    const uint32_t ans = lane_select<NMAX>(x, static_cast<uint32_t>(n), kth, lo, hi);
+    const bool split = hand != hor;  // this column's high words differ
+    if (mine && !split) m[w * RS + c0 + lane] = static_cast<int64_t>((static_cast<uint64_t>(hor) << 32) | ans);
+    for (uint32_t todo = __ballot_sync(kFull, mine && split); todo; todo &= todo - 1) {
+      const int64_t c = c0 + __ffs(todo) - 1;
+      const int64_t med = median_column_global<(NMAX + 31) / 32>(d + tb * RS + c, RS, n, hists[warp], lane);
+      if (lane == 0) m[w * RS + c] = med;
+    }
+  }
+}
+
+template <int NMAX>
+cudaError_t launch_median_lanes(const int64_t* d, int64_t T, int64_t RS, int64_t W, int64_t* m, cudaStream_t stream) {
+  const int64_t tiles = (RS + 31) / 32, ntiles = (T + W - 1) / W * tiles;
+  int per_sm = 0;
+  const cudaError_t e =
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, median_lanes_kernel<NMAX>, kLaneMedThreads, 0);
+  if (e != cudaSuccess) return e;
+  const int64_t warps = kLaneMedThreads / 32;
+  const int64_t grid = std::min<int64_t>((ntiles + warps - 1) / warps, int64_t(sm_count()) * std::max(per_sm, 1));
+  count_launch();
+  median_lanes_kernel<NMAX><<<static_cast<unsigned>(grid), kLaneMedThreads, 0, stream>>>(d, T, RS, W, tiles, ntiles, m);
+  return cudaGetLastError();
 }
 
 // Windows longer than 1024 steps: the same search, re-reading the column
@@ -773,7 +764,7 @@ template <int NPL>
 cudaError_t launch_median_npl(const int64_t* d, int64_t T, int64_t RS, int64_t W, int64_t nW,
                               int64_t ngroups, int64_t* m, cudaStream_t stream) {
   const size_t smem = size_t(kMedCols) * (32 * NPL + 1) * sizeof(int64_t) +
-                      size_t(kMedCols) * kMedBins * sizeof(uint32_t);
+                      size_t(kMedCols) * kSelBins * sizeof(uint32_t);
   const bool vec = (RS % 2) == 0 && (reinterpret_cast<uintptr_t>(d) % 16) == 0;
   auto kern = vec ? median_kernel<NPL, true> : median_kernel<NPL, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -787,7 +778,7 @@ cudaError_t launch_median_tma(const CUtensorMap& map, const int64_t* d, int64_t 
                               int64_t w0, int64_t nW, int64_t n, int64_t ngroups, int box_rows, int nbox, int64_t* m, uint32_t* status,
                               cudaStream_t stream) {
   const size_t tile_rows = std::max<size_t>(size_t(nbox) * box_rows, 32 * NPL);  // every slot's row is in the tile
-  const size_t smem = 1024 + tile_rows * 64 + size_t(kMedCols) * kMedHistWords * 4 + 32;  // + 2 mbarriers, flag
+  const size_t smem = 1024 + tile_rows * 64 + size_t(kMedCols) * kSelHistWords * 4 + 32;  // + 2 mbarriers, flag
   auto kern = n > 32 * (NPL - 1) ? median_persist_kernel<NPL, true> : median_persist_kernel<NPL, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
@@ -879,6 +870,14 @@ cudaError_t launch_window_median(const int64_t* d, int64_t T, int64_t R, int64_t
   const int64_t nW = (T + W - 1) / W;
   const int64_t ngroups = (RS + kMedCols - 1) / kMedCols;
   const int64_t n = std::min(W, T);
+  // (fewer tiles than four warps per SM: a warp per column spreads further, 48 columns
+  // by 10 windows 4.3 against 12.3 us)
+  if (n <= kLaneMedMaxRows && nW * ((RS + 31) / 32) >= int64_t(sm_count()) * 4) {
+    if (n <= 32) return launch_median_lanes<32>(d, T, RS, W, m, stream);
+    if (n <= 64) return launch_median_lanes<64>(d, T, RS, W, m, stream);
+    if (n <= 104) return launch_median_lanes<104>(d, T, RS, W, m, stream);
+    return launch_median_lanes<128>(d, T, RS, W, m, stream);
+  }
   // Bulk-copy path: rows of d are 16-byte multiples (RS even), d is 16-byte
   // aligned, windows fit the register path, the driver encoder is available.
   // A launch's windows share one row count (the slot tests depend on it), so

@@ -69,3 +69,34 @@ def test_gates_switches(sf, T, S, W):
 def test_ties_splits(sf, T, R, S):
     d_np = np.random.default_rng(T + R).integers(0, 4, size=(T, R, S)).astype(np.int64)
     assert np.array_equal(host(sf.sf_frontier_ties(dev(d_np))), O.frontier(d_np).ties)
+
+
+def durations(T, R, S, kind, seed):
+    """ms work; `long`: steps around 2^32 ns, where 32-bit row sums end; `far`:
+    one rank 2^31 ns and more from the others in some steps."""
+    rng = np.random.default_rng(seed)
+    d = np.rint(rng.uniform(1e6, 5e7, size=S) * np.exp(0.1 * rng.standard_normal((T, R, S)))).astype(np.int64)
+    if kind == "long":
+        total = d.sum(axis=2)
+        edge = (1 << 32) - 1 + rng.integers(-2, 3, size=(T, R))
+        pick = rng.random((T, R)) < 0.3
+        d[..., S - 1] += np.where(pick, edge - total, 0)
+    if kind == "far":
+        t = np.nonzero(rng.random(T) < 0.3)[0]
+        d[t, rng.integers(R, size=t.size), rng.integers(S, size=t.size)] += rng.integers(1 << 31, 1 << 34, size=t.size)
+    if kind == "tail":
+        d = np.rint(d * np.where(rng.random((T, R, 1)) < 0.01, 30.0, 1.0)).astype(np.int64)
+    return d
+
+
+# windows whose columns single lanes hold: rows of each form and one more, a
+# short last window, odd column counts, columns with one far value among them
+@pytest.mark.parametrize("T,R,S,W", [(70, 3, 5, 16), (33, 7, 3, 32), (100, 5, 7, 33), (128, 31, 1, 64), (200, 9, 9, 65),
+                                     (305, 11, 8, 100), (210, 33, 4, 104), (300, 13, 3, 105), (257, 16, 2, 128),
+                                     (260, 16, 2, 129)])
+@pytest.mark.parametrize("kind", ["ms", "far", "tail", "few"])
+def test_median_lanes(sf, T, R, S, W, kind):
+    d_np = durations(T, R, S, kind, T + W)
+    if kind == "few":
+        d_np = np.random.default_rng(T).integers(0, 3, size=(T, R, S)).astype(np.int64) - 1
+    assert np.array_equal(host(sf.sf_window_median(dev(d_np), W)), O.window_median(d_np, W))
