@@ -3,7 +3,8 @@
 // durations d[t,r,s] (for the raw rank spread of the Sec. 6 routing table),
 // with the maximum and the second largest value.
 //
-// The steps are processed in chunks whose scratch stays in L2; per chunk two
+// Steps whose keys fit one SM are selected there (sf_rank_chip.cu); this file
+// takes the larger ones.  They are processed in chunks whose scratch stays in L2; per chunk two
 // kernels run, the encode of the next chunk overlapping the select of this
 // one (programmatic dependent launch, two scratch buffers):
 //  encode (rank_encode_split_kernel for 4, 8 or 16 stages, a rank row split
@@ -827,6 +828,7 @@ cudaError_t launch_rank_select(const int64_t* d, int64_t T, int64_t R, int64_t S
                                int64_t W, int64_t* L, int64_t* dL, int64_t* G, int64_t* Lw, int64_t* Gw,
                                int64_t* spread, void* workspace, size_t ws_bytes, uint32_t* status,
                                cudaStream_t stream) {
+  if (rank_on_chip(R, S)) return launch_rank_chip(d, T, R, S, of_prefix, t0, W, L, dL, G, Lw, Gw, spread, status, stream);
   const size_t half = ws_bytes / 2 & ~size_t(255);  // one chunk buffer, 256-byte aligned
   const int64_t Tc = chunk_steps_for(T, R, S, half);
   if (Tc < 1) return cudaErrorInvalidValue;

@@ -100,3 +100,29 @@ def test_median_lanes(sf, T, R, S, W, kind):
     if kind == "few":
         d_np = np.random.default_rng(T).integers(0, 3, size=(T, R, S)).astype(np.int64) - 1
     assert np.array_equal(host(sf.sf_window_median(dev(d_np), W)), O.window_median(d_np, W))
+
+
+# steps held on chip: keys per lane, per warp, the CTA form's columns in registers
+# and in shared memory, the first ranks past each, columns in which every key falls
+# into a few bins, and medians on both sides of the bracket
+@pytest.mark.parametrize("T,R,S", [(40, 1, 4), (1, 1, 1), (40, 2, 2), (30, 32, 17), (30, 33, 17), (30, 64, 9), (30, 65, 16),
+                                   (30, 128, 8), (30, 129, 8), (20, 256, 3), (20, 257, 4), (9, 1024, 2),
+                                   (9, 4099, 1), (7, 1001, 13), (7, 2893, 8), (7, 2945, 8), (5, 700, 32),
+                                   (40, 16, 8), (41, 17, 16), (30, 104, 10), (30, 105, 5), (33, 128, 32), (7, 2048, 9),
+                                   (5, 2049, 1), (5, 2050, 2), (6, 2051, 3), (5, 4097, 5), (4, 8192, 8), (3, 9001, 16),
+                                   (2, 16385, 12), (2, 32768, 8), (2, 4500, 32), (1, 65536, 8), (300, 3000, 4)])
+@pytest.mark.parametrize("kind", ["ms", "long", "far", "tail", "halves"])
+def test_rank_on_chip(sf, T, R, S, kind):
+    d_np = durations(T, R, S, kind, T + R + S)
+    if kind == "halves":  # ranks split into two far groups, lane by lane: empty and misleading brackets
+        d_np[:, np.arange(R) % 32 < (R + S) % 32, 0] *= 9
+    o = O.rank_lag(d_np)
+    st = sf.new_status("cuda")
+    g = sf.sf_rank_lag(dev(d_np), status=st)
+    sp = sf.sf_raw_spread(dev(d_np), 4, t0=3, status=st)
+    Lw, Gw = sf.sf_rank_lag_windows(dev(d_np), 4, t0=3, status=st)
+    oL, oG = O.rank_lag_windows(d_np, 4, 3)
+    assert int(st.item()) == 0
+    assert np.array_equal(host(g.L), o.L) and np.array_equal(host(g.dL), o.dL) and np.array_equal(host(g.G), o.G)
+    assert np.array_equal(host(sp), O.raw_spread(d_np, 4, 3))
+    assert np.array_equal(host(Lw), oL) and np.array_equal(host(Gw), oG)
