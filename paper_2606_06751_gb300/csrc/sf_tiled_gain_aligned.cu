@@ -1,0 +1,11 @@
+// sf_tiled_gain_aligned.cu - the tiled evidence pass, steps of whole 128-byte rows.
+#include "sf_tiled.cuh"
+
+namespace sf {
+
+cudaError_t launch_gain_aligned(const CUtensorMap& map, const CUtensorMap& map_m, const Params& p, int grid,
+                                cudaStream_t stream, bool pdl) {
+  return dispatch_tiled<kGain, true>(map, map_m, p, grid, stream, pdl);
+}
+
+}  // namespace sf

@@ -126,3 +126,43 @@ def test_rank_on_chip(sf, T, R, S, kind):
     assert np.array_equal(host(g.L), o.L) and np.array_equal(host(g.dL), o.dL) and np.array_equal(host(g.G), o.G)
     assert np.array_equal(host(sp), O.raw_spread(d_np, 4, 3))
     assert np.array_equal(host(Lw), oL) and np.array_equal(host(Gw), oG)
+
+
+# steps that are not whole 128-byte rows: every stage count, small steps (whole
+# steps per tile) and steps of one or more tiles with one, two and four warp
+# groups, a tensor and medians that end inside a row, tensors below one row;
+# then whole-row steps around the limits between those forms
+TILED = [(300, 31, 1, 70), (4000, 3, 2, 500), (200, 61, 3, 33), (50, 127, 4, 20), (90, 201, 5, 40), (33, 97, 6, 11),
+         (500, 31, 7, 64), (40, 101, 8, 9), (77, 63, 9, 30), (31, 85, 10, 16), (64, 55, 11, 20), (25, 99, 12, 7),
+         (80, 41, 13, 33), (22, 73, 14, 10), (45, 67, 15, 13), (3, 5, 1, 2), (1, 1, 1, 1), (2000, 1, 5, 300),
+         (9, 9001, 1, 4), (7, 5001, 2, 3), (11, 1001, 3, 4), (9, 2001, 4, 4), (13, 1000, 5, 6), (8, 700, 6, 3),
+         (10, 601, 7, 4), (9, 1001, 8, 4), (7, 2003, 9, 3), (6, 1701, 10, 4), (8, 333, 11, 3), (9, 501, 12, 5),
+         (6, 2001, 13, 2), (7, 403, 14, 3), (5, 1555, 15, 2), (4, 32767, 3, 2),
+         (40, 128, 8, 15), (40, 130, 8, 15), (30, 64, 16, 12), (12, 512, 8, 5), (12, 514, 8, 5), (9, 2048, 8, 4),
+         (9, 96, 14, 4), (20, 192, 10, 6), (7, 1024, 16, 3)]
+
+
+@pytest.mark.parametrize("T,R,S,W", TILED)
+@pytest.mark.parametrize("kind", ["ms", "long"])
+def test_tiled_passes(sf, T, R, S, W, kind):
+    d_np = durations(T, R, S, kind, T + R + S)
+    d, st = dev(d_np), sf.new_status("cuda")
+    f, o = sf.sf_frontier(d, status=st), O.frontier(d_np)
+    assert np.array_equal(host(f.a), o.a) and np.array_equal(host(f.lead), o.lead)
+    assert np.array_equal(host(f.makespan), o.makespan)
+    win, ow = sf.sf_window_aggregate(d, W, t0=1, status=st), O.windows(d_np, W, 1)
+    assert np.array_equal(host(win.X), ow.X) and np.array_equal(host(win.E), ow.E)
+    assert np.array_equal(host(win.C), ow.C) and np.array_equal(host(win.step_lead), ow.step_lead)
+    b, ob = sf.sf_window_baselines(d, W, status=st), O.baselines(d_np, W)
+    assert np.array_equal(host(b.M), ob.M) and np.array_equal(host(b.SLOW), ob.SLOW)
+    assert np.array_equal(host(b.RANK0), ob.RANK0)
+    assert np.array_equal(host(b.SUM.view(torch.int64))[..., 0], ob.SUM.astype(np.int64))
+    m_np = O.window_median(d_np, W)
+    ev, ow = sf.sf_direct_gain(d, W, dev(m_np), lead_credit=True, status=st), O.windows(d_np, W)
+    assert np.array_equal(host(ev.X), ow.X) and np.array_equal(host(ev.Y), O.direct_gain(d_np, W, m_np))
+    assert np.array_equal(host(ev.E), ow.E) and np.array_equal(host(ev.C), ow.C)
+    wall = d_np.sum(axis=2) + 1000
+    lab = sf.sf_label_windows(d, W, wall=dev(wall), other_stage=S - 1, status=st)
+    ol = O.label_windows(d_np, W, wall=wall, other_stage=S - 1)
+    assert np.array_equal(host(lab.labels).astype(np.uint32), ol.labels) and np.array_equal(host(lab.Y), ol.Y)
+    assert int(st.item()) == 0
