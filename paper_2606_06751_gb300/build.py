@@ -18,7 +18,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(PKG, "libstagefrontier.so")
 SOURCES = [*(f"sf_tiled_{kind}_{steps}.cu" for kind in ("quality", "gain", "base", "frontier")
-             for steps in ("unaligned", "aligned")), "sf_lanes.cu", "sf_stream.cu",
+             for steps in ("unaligned", "aligned")), "sf_lanes.cu", "sf_step_lanes.cu", "sf_stream.cu",
            "sf_select.cu", "sf_rank.cu", "sf_rank_chip.cu", "sf_rank_lanes.cu", "sf_rank_warp.cu", "sf_group.cu",
            "sf_ingest.cu", "sf_api.cu", "sf_static.cu", "sf_pipeline.cu", "sf_ties.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -478,6 +478,21 @@ EncodeFn encode_fn() {
 
 namespace {
 
+// One lane per (step, stage) instead of tiles: small steps, whose S warp
+// reductions each outweigh their few rank rows, and the evidence pass over more
+// stages than the tiles take.  Measured on 0.1 to 1.1 GB, tiles against lanes, us:
+// evidence 16 x 8 88 / 39, 64 x 16 422 / 269, 64 x 8 115 / 111, 128 x 16 111 / 95,
+// 128 x 8 164 / 202, 256 x 8 239 / 246; baselines 64 x 8 114 / 88, 128 x 8 144 / 164;
+// frontier 12 x 3 133 / 38, 31 x 7 61 / 47, 128 x 6 102 / 131; evidence 1000 x 24
+// 570 (a CTA per step) / 183.  The warps (20 per SM) need steps enough to go round.
+bool use_step_lanes(int kind, int64_t T, int64_t R, int64_t S, bool fast, int sms) {
+  if (S <= 16 && !fast) return T >= int64_t(sms) * 32;  // medians only 8-byte aligned
+  if ((T + 32 / S - 1) / (32 / S) < int64_t(sms) * 4) return false;
+  if (kind == kFrontier) return S <= 16 && lanes_groups(R, S) == 0 && R * S * 8 <= 3072;
+  if (S > 16) return is_gain(kind);
+  return R <= 64 || (S == 16 && R <= 128);
+}
+
 // Whether the evidence pass keeps whole windows of medians (`rows` 128-byte
 // rows each) in shared memory, and how.  Two slots let a window's copy run
 // under the steps of the one before; one slot stands idle for a copy at each
@@ -565,6 +580,10 @@ cudaError_t launch_stream_pass(const StreamJob& j, cudaStream_t stream) {
     return e;
   }
   const int kind = j.gain ? (j.quality ? kGainQuality : kGain) : j.base ? kBase : kFrontier;
+  if (use_step_lanes(kind, j.T, j.R, j.S, fast, sms)) {
+    count_launch();
+    return launch_step_lanes(kind, p, stream, j.after_clear);
+  }
   if (fast) {
     const bool gain = j.gain;
     const int warps = consumer_warps(kind, j.S);

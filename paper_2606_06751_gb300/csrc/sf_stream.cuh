@@ -83,6 +83,8 @@ using TiledLaunch = cudaError_t(const CUtensorMap& map, const CUtensorMap& map_m
                                 cudaStream_t stream, bool pdl);
 TiledLaunch launch_frontier_aligned, launch_frontier_unaligned, launch_gain_aligned, launch_gain_unaligned,
     launch_quality_aligned, launch_quality_unaligned, launch_base_aligned, launch_base_unaligned;
+// one lane per (step, stage)
+cudaError_t launch_step_lanes(int kind, const Params& p, cudaStream_t stream, bool pdl);
 // several steps per warp instruction: lanes_groups is their number G, 0 where the shape takes one
 int lanes_groups(int64_t R, int64_t S);
 cudaError_t launch_lanes(int G, const CUtensorMap& map, const Params& p, int grid, cudaStream_t stream, bool pdl);
