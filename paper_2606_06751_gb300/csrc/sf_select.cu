@@ -5,6 +5,7 @@
 //   * gates: App. C label gates, routing and ambiguity sets, fp64 shares/gains;
 //   * zero: clears accumulators the library owns the semantics of.
 #include <algorithm>
+#include <type_traits>
 
 #include <cooperative_groups.h>
 
@@ -202,6 +203,45 @@ __device__ __noinline__ int64_t median_column_global(const int64_t* __restrict__
   return static_cast<int64_t>(key ^ kSign);
 }
 
+// A column of the tile whose values do not share their high words, most often
+// for a few outliers alone (one stall of seconds among milliseconds): row 0's
+// high word is tried for the median's.  Larger values become the largest of the
+// column that share it, smaller ones the smallest, in the tile, which moves the
+// median only if it is not among the sharers; returns false, with the tile as it
+// was, if it is not.  row0: the column's place in the tile's first row.
+__device__ __noinline__ bool clamp_column(unsigned char* row0, uint32_t swizzle_bits, int n, int lane) {
+  // rows are 64 bytes apart, their 16-byte chunks permuted by bits 1-2 of the row
+  auto at = [&](int r) {
+    return reinterpret_cast<uint2*>(row0 + r * 64 + (((swizzle_bits >> 1) ^ ((r >> 1) & 3)) << 4) + ((swizzle_bits & 1) << 3));
+  };
+  const uint32_t h0 = at(0)->y, k = static_cast<uint32_t>((n - 1) / 2);
+  uint32_t same = 0, under = 0, lo = 0xffffffffu, hi = 0;
+#pragma unroll 4
+  for (int r = lane; r < n; r += 32) {
+    const uint2 v = *at(r);
+    if (v.y == h0) {
+      ++same;
+      lo = min(lo, v.x);
+      hi = max(hi, v.x);
+    } else if (static_cast<int32_t>(v.y) < static_cast<int32_t>(h0)) {
+      ++under;
+    }
+  }
+  same = __reduce_add_sync(kFull, same);
+  under = __reduce_add_sync(kFull, under);
+  if (k < under || k - under >= same) return false;
+  lo = __reduce_min_sync(kFull, lo);
+  hi = __reduce_max_sync(kFull, hi);
+#pragma unroll 4
+  for (int r = lane; r < n; r += 32) {
+    const uint2 v = *at(r);
+    if (v.y != h0) *at(r) = make_uint2(static_cast<int32_t>(v.y) < static_cast<int32_t>(h0) ? lo : hi, h0);
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // before the next tile's copies
+  __syncwarp();
+  return true;
+}
+
 // Persistent form of the median: each CTA walks (window, 8-column) tiles
 // with one tile buffer and two mbarriers.  `full` completes when a tile's
 // bulk copies have landed; each warp copies its column into registers and
@@ -209,8 +249,10 @@ __device__ __noinline__ int64_t median_column_global(const int64_t* __restrict__
 // of the CTA's next tile into the same buffer, so the copy runs under the
 // selection of the current tile and no CTA-wide barrier aligns the warps.
 // The selection touches only registers and the warp's counters.  A column
-// whose values do not share their high 32 bits selects on 64-bit values
-// re-read from d.  Every window of a launch holds the same n rows.
+// whose median is not among the values that share row 0's high 32 bits selects
+// on 64-bit values re-read from d (all columns with an outlier past 32 bits did:
+// a heavy-tailed 50000 x 1024 x 10, W = 500, 1352 us); past 512 rows, any column
+// whose values do not share them.  Every window of a launch holds the same n rows.
 //
 // Resident CTAs hide each tile's copy and selection chain, so the registers are
 // held to what the most CTAs allow without spilling the column (512-row columns,
@@ -232,10 +274,14 @@ __global__ void __launch_bounds__(kMedThreads, med_min_ctas(NPL))
   volatile int* abort = reinterpret_cast<volatile int*>(full + 2);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint32_t* hist = hists + warp * kSelHistWords;
-  const int64_t ntiles = nW * ngroups;
-  auto issue = [&](int64_t id) {  // one thread: the bulk copies of tile `id`
-    const int64_t c0 = (id % ngroups) * kMedCols;
-    const int64_t tb = (w0 + id / ngroups) * W;
+  // Tile numbers, columns of a step and windows of a launch fit 32 bits (the entry
+  // point's limits): shorter divisions, fewer registers (512 rows: 824 -> 803 us).
+  // With 32 slots that made the compiler spill the column, twice the time.
+  using Id = std::conditional_t<(NPL > 16), int64_t, uint32_t>;
+  const Id groups = static_cast<Id>(ngroups), ntiles = static_cast<Id>(nW) * groups;
+  auto issue = [&](Id id) {  // one thread: the bulk copies of tile `id`
+    const Id c0 = (id % groups) * kMedCols;
+    const int64_t tb = (w0 + id / groups) * W;
     mbar_arrive_expect_tx(full, tile_bytes);
     for (int b = 0; b < nbox; ++b)
       tma_load_2d(tile + size_t(b) * box_rows * 64, &map, static_cast<int32_t>(c0),
@@ -252,9 +298,9 @@ __global__ void __launch_bounds__(kMedThreads, med_min_ctas(NPL))
   if (threadIdx.x == 0 && issued) issue(blockIdx.x);
   const unsigned char* col = tile + lane * 64u + ((((warp >> 1) ^ ((lane >> 1) & 3)) << 4) | ((warp & 1) << 3));
   uint32_t phase = 0;
-  for (int64_t id = blockIdx.x; id < ntiles; id += gridDim.x, phase ^= 1u) {
-    const int64_t w = w0 + id / ngroups;
-    const int64_t c0 = (id % ngroups) * kMedCols;
+  for (Id id = blockIdx.x; id < ntiles; id += gridDim.x, phase ^= 1u) {
+    const int64_t w = w0 + id / groups;
+    const Id c0 = (id % groups) * kMedCols;
     const bool mine = warp < imin64(kMedCols, RS - c0);
     const int n = static_cast<int>(imin64(W, T - w * W));
     // a warp goes on only if all its lanes saw the tile (a wait gives up
@@ -271,19 +317,28 @@ __global__ void __launch_bounds__(kMedThreads, med_min_ctas(NPL))
     // high words agree iff their AND equals their OR over the column.
     auto live = [&](int i) { return (kFit && i + 1 < NPL) || lane + 32 * i < n; };
     uint32_t xl[NPL];
-    uint32_t hand = 0xffffffffu, hor = 0u, live_x = 0u;
+    uint32_t hand, hor, live_x = 0u;
+    for (bool again = NPL <= 16 && mine;; again = false) {
+      hand = 0xffffffffu;
+      hor = 0u;
 #pragma unroll
-    for (int i = 0; i < NPL; ++i) {
-      const uint2 v = *reinterpret_cast<const uint2*>(col + i * 2048);  // in the tile even past the window
-      if (i == 0) live_x = kFit && NPL >= 2 ? v.x : __shfl_sync(kFull, v.x, 0);  // row 0 is in every window
-      const bool okr = live(i);
-      xl[i] = okr ? v.x : live_x;
-      hand &= okr ? v.y : 0xffffffffu;
-      hor |= okr ? v.y : 0u;
+      for (int i = 0; i < NPL; ++i) {
+        const uint2 v = *reinterpret_cast<const uint2*>(col + i * 2048);  // in the tile even past the window
+        if (i == 0) live_x = kFit && NPL >= 2 ? v.x : __shfl_sync(kFull, v.x, 0);  // row 0 is in every window
+        const bool okr = live(i);
+        xl[i] = okr ? v.x : live_x;
+        hand &= okr ? v.y : 0xffffffffu;
+        hor |= okr ? v.y : 0u;
+      }
+      // a column whose high words differ is clamped and read once more (not with 32
+      // slots: the call's registers would spill them)
+      if (NPL > 16 || !again || __reduce_and_sync(kFull, hand) == __reduce_or_sync(kFull, hor) ||
+          !clamp_column(tile, static_cast<uint32_t>(warp), n, lane))
+        break;
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(empty);  // this warp is done with the buffer
-    const int64_t next = id + gridDim.x;
+    const Id next = id + gridDim.x;
     if (threadIdx.x == 0 && next < ntiles) {
       issued = mbar_wait_bounded(empty, phase, abort);
       if (issued) issue(next);  // else the abort flag is set and every warp leaves at its next wait

@@ -89,14 +89,22 @@ def durations(T, R, S, kind, seed):
     return d
 
 
-# windows whose columns single lanes hold: rows of each form and one more, a
-# short last window, odd column counts, columns with one far value among them
+# windows whose columns single lanes hold (where they are enough) and longer ones:
+# rows of each form and one more, a short last window, odd column counts, columns
+# whose values differ in their high words
 @pytest.mark.parametrize("T,R,S,W", [(70, 3, 5, 16), (33, 7, 3, 32), (100, 5, 7, 33), (128, 31, 1, 64), (200, 9, 9, 65),
                                      (305, 11, 8, 100), (210, 33, 4, 104), (300, 13, 3, 105), (257, 16, 2, 128),
-                                     (260, 16, 2, 129)])
-@pytest.mark.parametrize("kind", ["ms", "far", "tail", "few"])
+                                     (260, 16, 2, 129), (305, 200, 20, 100), (1000, 40, 2, 250), (1001, 6, 4, 500),
+                                     (2000, 5, 2, 1000), (700, 3, 3, 300)])
+@pytest.mark.parametrize("kind", ["ms", "far", "tail", "few", "words"])
 def test_median_lanes(sf, T, R, S, W, kind):
     d_np = durations(T, R, S, kind, T + W)
+    if kind == "words":  # most values share a high word, a few lie above and below, in row 0 of some columns too
+        rng = np.random.default_rng(T)
+        d_np += 1 << 32
+        d_np[rng.random(d_np.shape) < 0.02] += 1 << 33
+        d_np[rng.random(d_np.shape) < 0.02] -= 1 << 32
+        d_np[0, ::3] += 1 << 33
     if kind == "few":
         d_np = np.random.default_rng(T).integers(0, 3, size=(T, R, S)).astype(np.int64) - 1
     assert np.array_equal(host(sf.sf_window_median(dev(d_np), W)), O.window_median(d_np, W))
