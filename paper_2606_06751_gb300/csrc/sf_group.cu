@@ -12,10 +12,19 @@
 // issues its own.  The per-group increments F_g[s] - F_g[s-1] and makespans
 // then accumulate in shared memory per window and are added to global memory
 // once per window the CTA touches.
+//
+// group_lanes_kernel: steps of few ranks, one lane per (step, stage).  Three CTA
+// barriers and a shared atomic per warp and stage are most of a small step's time
+// above; here a warp walks the ranks of 32 / S consecutive steps together, each
+// lane keeping the running maximum of the rank's group for its own stage and
+// parking it in shared memory when the group changes, so no lane waits for
+// another before the step's end.
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "sf_device.cuh"
+#include "sf_lane_select.cuh"
 #include "sf_launch.h"
 
 namespace sf {
@@ -172,6 +181,150 @@ __global__ void __launch_bounds__(kGrThreads) group_window_kernel(const GroupPar
   if (lane == 0) report(p.status, bits);
 }
 
+// ---------------------------------------------------------------- few ranks
+
+constexpr int kGlThreads = 128;
+constexpr int kGlWarps = kGlThreads / 32;
+constexpr int kGlBatch = 8;
+constexpr int kGlMaxGroups = 32;
+// (us, CTA per step / lanes: 100000 x 16 x 8 461 / 72, 100000 x 31 x 7 563 / 82,
+// 131072 x 64 x 16 753 / 309, 100000 x 128 x 8 352 / 254, 50000 x 300 x 6 237 / 271)
+constexpr int64_t kGlMaxRanks = 192;
+
+// Walks the ranks of a warp's steps: park[g][lane] becomes the lane's stage of
+// F_g.  32-bit prefixes unless WIDE; returns whether they hold.
+template <int LOGS, bool WIDE>
+__device__ __forceinline__ bool group_walk(const GroupParams& p, const int64_t* col, int s, uint64_t* park, int lane,
+                                           uint32_t& dor, uint32_t& tor, uint32_t& bad_group) {
+  using V = std::conditional_t<WIDE, uint64_t, uint32_t>;
+  const int R = static_cast<int>(p.R), S = static_cast<int>(p.S), G = static_cast<int>(p.G);
+  for (int g = 0; g < G; ++g) park[g * 32 + lane] = 0;
+  uint32_t vmax = 0, dhi = 0;
+  V best = 0;
+  int cur = -1;  // the group `best` belongs to, the same in every lane
+  for (int r0 = 0; r0 < R; r0 += kGlBatch) {
+    uint2 v[kGlBatch];
+    int32_t gr[kGlBatch];
+#pragma unroll
+    for (int i = 0; i < kGlBatch; ++i) {
+      const int r = min(r0 + i, R - 1);  // past the ranks: the last one again, which changes no maximum
+      v[i] = load_words(col + int64_t(r) * S);
+      gr[i] = __ldg(p.group + r);
+    }
+#pragma unroll
+    for (int i = 0; i < kGlBatch; ++i) {
+      const V y = WIDE ? static_cast<V>((static_cast<uint64_t>(v[i].y) << 32) | v[i].x) : static_cast<V>(v[i].x);
+      const bool ok = gr[i] >= 0 && gr[i] < G;
+      bad_group |= ok ? 0u : 1u;
+      V P = ok ? y : V(0);
+      if (ok) {
+        dhi |= v[i].y;
+        vmax = max(vmax, v[i].x);
+      }
+#pragma unroll
+      for (int q = 1; q < (1 << LOGS); q <<= 1) {
+        const V up = __shfl_up_sync(kFull, P, q);
+        if (s >= q) P += up;
+      }
+      if constexpr (WIDE)
+        if (s == S - 1) tor |= static_cast<uint32_t>(static_cast<uint64_t>(P) >> 32);
+      if (ok && gr[i] != cur) {
+        if (cur >= 0) park[cur * 32 + lane] = best;
+        cur = gr[i];
+        best = static_cast<V>(park[cur * 32 + lane]);
+      }
+      if (ok) best = WIDE ? (static_cast<int64_t>(P) > static_cast<int64_t>(best) ? P : best) : (P > best ? P : best);
+    }
+  }
+  if (cur >= 0) park[cur * 32 + lane] = best;
+  if constexpr (WIDE) dor |= dhi;
+  uint64_t bound = dhi ? uint64_t(1) << 32 : vmax;  // the lanes' largest values bound the prefixes
+#pragma unroll
+  for (int q = 1; q < (1 << LOGS); q <<= 1) {
+    const uint64_t up = __shfl_up_sync(kFull, bound, q);
+    if (s >= q) bound += up;
+  }
+  return (bound >> 32) == 0;
+}
+
+template <int LOGS>
+__device__ __noinline__ bool group_walk_wide(const GroupParams& p, const int64_t* col, int s, uint64_t* park, int lane,
+                                             uint32_t& dor, uint32_t& tor, uint32_t& bad_group) {
+  return group_walk<LOGS, true>(p, col, s, park, lane, dor, tor, bad_group);
+}
+
+template <int LOGS>
+__global__ void __launch_bounds__(kGlThreads, 5) group_lanes_kernel(const __grid_constant__ GroupParams p) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int S = static_cast<int>(p.S), G = static_cast<int>(p.G);
+  uint64_t* park = reinterpret_cast<uint64_t*>(dyn) + size_t(warp) * 2 * G * 32;  // [G][32]
+  int64_t* acc = reinterpret_cast<int64_t*>(park + G * 32);                       // [G][32] the lane's window sums
+  const int steps = 32 / S, j = lane / S, s = lane - j * S;
+  const int64_t tiles = (p.T + steps - 1) / steps;
+  const int64_t nw = int64_t(gridDim.x) * kGlWarps, id = int64_t(blockIdx.x) * kGlWarps + warp;
+  const int64_t tile_end = tiles * (id + 1) / nw;
+  uint32_t dor = 0, tor = 0, bad_group = 0;
+  int64_t w = -1, w_end = 0;  // window of the lane's step: steps below w_end
+  bool wide = false;          // walk the next tile in 64 bits at once
+  for (int g = 0; g < G; ++g) acc[g * 32 + lane] = 0;
+  auto flush = [&]() {
+    if (w < 0) return;
+    for (int g = 0; g < G; ++g) {
+      const int64_t x = acc[g * 32 + lane];
+      if (x == 0) continue;
+      acc[g * 32 + lane] = 0;
+      atomicAdd(reinterpret_cast<unsigned long long*>(&p.Xg[(w * G + g) * S + s]), static_cast<unsigned long long>(x));
+      // the increments of a step add up to its makespan
+      atomicAdd(reinterpret_cast<unsigned long long*>(&p.Dg[w * G + g]), static_cast<unsigned long long>(x));
+    }
+  };
+  for (int64_t tile = tiles * id / nw; tile < tile_end; ++tile) {
+    const int64_t t0 = tile * steps;
+    const bool live = j < steps && t0 + j < p.T;
+    const int64_t t = live ? t0 + j : t0;
+    if (live && (w < 0 || t >= w_end)) {
+      flush();
+      w = (p.t0 + t) / p.W - p.w_first;
+      w_end = (w + p.w_first + 1) * p.W - p.t0;
+    }
+    const int64_t* col = p.d + t * p.R * S + s;
+    bool fits;
+    if (!wide) {
+      fits = group_walk<LOGS, false>(p, col, s, park, lane, dor, tor, bad_group);
+      wide = !__all_sync(kFull, fits);
+      if (wide) group_walk_wide<LOGS>(p, col, s, park, lane, dor, tor, bad_group);
+    } else {
+      fits = group_walk_wide<LOGS>(p, col, s, park, lane, dor, tor, bad_group);
+      wide = !__all_sync(kFull, fits);
+    }
+    for (int g = 0; g < G; ++g) {
+      const int64_t F = static_cast<int64_t>(park[g * 32 + lane]);
+      const int64_t before = __shfl_up_sync(kFull, F, 1);
+      if (live) acc[g * 32 + lane] += F - (s ? before : 0);
+    }
+  }
+  flush();
+  uint32_t bits = range_bits(__reduce_or_sync(kFull, dor), __reduce_or_sync(kFull, tor));
+  if (__any_sync(kFull, bad_group != 0)) bits |= SF_ST_INDEX;
+  if (lane == 0) report(p.status, bits);
+}
+
+template <int LOGS>
+cudaError_t launch_group_lanes(const GroupParams& p, cudaStream_t stream) {
+  auto kern = group_lanes_kernel<LOGS>;
+  const size_t smem = size_t(kGlWarps) * 2 * p.G * 32 * 8;  // at most 64 KB
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  int per_sm = 0;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGlThreads, smem);
+  if (e != cudaSuccess) return e;
+  const int64_t tiles = (p.T + 32 / p.S - 1) / (32 / p.S);
+  const int64_t grid = std::min<int64_t>((tiles + kGlWarps - 1) / kGlWarps, int64_t(sm_count()) * std::max(per_sm, 1));
+  count_launch();
+  kern<<<static_cast<unsigned>(grid), kGlThreads, smem, stream>>>(p);
+  return cudaGetLastError();
+}
+
 struct StageGroups {
   int32_t of[32];  // stage -> reporting group
 };
@@ -223,6 +376,14 @@ cudaError_t launch_group_windows(const int64_t* d, int64_t T, int64_t R, int64_t
   p.Xg = Xg;
   p.Dg = Dg;
   p.status = status;
+  if (R <= kGlMaxRanks && G <= kGlMaxGroups && (T + 32 / S - 1) / (32 / S) >= int64_t(sm_count()) * 4) {
+    if (S <= 1) return launch_group_lanes<0>(p, stream);
+    if (S <= 2) return launch_group_lanes<1>(p, stream);
+    if (S <= 4) return launch_group_lanes<2>(p, stream);
+    if (S <= 8) return launch_group_lanes<3>(p, stream);
+    if (S <= 16) return launch_group_lanes<4>(p, stream);
+    return launch_group_lanes<5>(p, stream);
+  }
   const size_t smem = size_t(G) * S * 16 + size_t(G) * 8;
   switch (S) {
     case 4: return launch_group_t<4>(p, smem, stream);

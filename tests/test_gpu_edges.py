@@ -174,3 +174,22 @@ def test_tiled_passes(sf, T, R, S, W, kind):
     ol = O.label_windows(d_np, W, wall=wall, other_stage=S - 1)
     assert np.array_equal(host(lab.labels).astype(np.uint32), ol.labels) and np.array_equal(host(lab.Y), ol.Y)
     assert int(st.item()) == 0
+
+
+# few ranks: a lane per (step, stage), every scan depth, one to 32 groups in blocks
+# and in any order, a group without ranks, the last rank count and one more, steps
+# past 32 bits, a partial last tile and window
+@pytest.mark.parametrize("T,R,S,G", [(20000, 7, 1, 2), (10001, 9, 2, 3), (5000, 40, 4, 1), (4001, 33, 7, 5),
+                                     (2600, 65, 8, 32), (2001, 50, 13, 4), (1300, 192, 16, 3), (1300, 193, 16, 3),
+                                     (700, 20, 24, 6), (650, 12, 32, 2)])
+@pytest.mark.parametrize("kind", ["blocks", "mixed", "long"])
+def test_group_lanes(sf, T, R, S, G, kind):
+    d_np = durations(T, R, S, "long" if kind == "long" else "ms", T + R)
+    rng = np.random.default_rng(T)
+    group = np.sort(rng.integers(0, max(1, G - 1), size=R)) if kind == "blocks" else rng.integers(0, G, size=R)
+    group = group.astype(np.int32)
+    o = O.group_windows(d_np, group, G, 100, 3)
+    st = sf.new_status("cuda")
+    g = sf.sf_group_aggregate(dev(d_np), dev(group), G, 100, t0=3, status=st)
+    assert int(st.item()) == 0
+    assert np.array_equal(host(g.X), np.transpose(o.X, (1, 0, 2))) and np.array_equal(host(g.D), o.D.T)
