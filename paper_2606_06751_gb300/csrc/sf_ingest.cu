@@ -41,10 +41,77 @@ __global__ void __launch_bounds__(kIngThreads) gathered_to_steps_kernel(const in
   }
 }
 
+// Through shared memory: tiles of kTileSteps steps of one window by as many
+// ranks as fit, so that both sides move in runs (a rank's kTileSteps S values in,
+// a step's ranks x S values out) where the kernel above reads S values at a time
+// and gives a whole CTA to a step.  A warp moves one run at a time, 8 bytes a lane
+// (16 bytes a lane read slower: fewer lanes per run, more registers).
+constexpr int kTileSteps = 16;
+constexpr int kTileBytes = 48 * 1024;
+
+// values of a rank's run in the tile, padded to an odd number against bank conflicts
+__host__ __device__ constexpr int tile_pitch(int S) { return kTileSteps * S | 1; }
+
+// Steps a CTA has little to do for (us before and with tiles: 100000 x 16 x 8 102 /
+// 45, 100000 x 31 x 7 161 / 90); larger ones move as fast or faster directly
+// (100000 x 128 x 8 262 / 292, 13421 x 1000 x 5 230 / 235, 8192 x 8 358 / 371).
+bool use_tiles(int64_t R, int64_t S, int64_t N) { return N >= kTileSteps && R * S * 8 <= 3072; }
+
+__global__ void __launch_bounds__(kIngThreads) gathered_tiles_kernel(const int64_t* __restrict__ src, int64_t T,
+                                                                     int64_t R, int S, int64_t N, int ranks,
+                                                                     int64_t* __restrict__ dst) {
+  __shared__ int64_t tile[kTileBytes / 8];  // [ranks][pitch]
+  constexpr int kWarps = kIngThreads / 32;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int pitch = tile_pitch(S);
+  const int step_r = 32 / S, step_s = 32 - step_r * S;  // a lane's next value of a step: ranks on, stages on
+  const int64_t per_window = (N + kTileSteps - 1) / kTileSteps, windows = (T + N - 1) / N;
+  const int64_t blocks = (R + ranks - 1) / ranks, tiles = windows * per_window * blocks;
+  for (int64_t id = blockIdx.x; id < tiles; id += gridDim.x) {
+    const int64_t b = id % blocks, q = id / blocks;
+    const int64_t win = q / per_window, t0 = (q - win * per_window) * kTileSteps;
+    const int64_t nb = min(N, T - win * N);
+    if (t0 >= nb) continue;  // the last window may be short
+    const int steps = static_cast<int>(min(int64_t(kTileSteps), nb - t0));
+    const int64_t r0 = b * ranks;
+    const int nr = static_cast<int>(min(int64_t(ranks), R - r0));
+    const int64_t* from = src + win * N * R * S + (r0 * nb + t0) * S;
+    const int run = steps * S;
+#pragma unroll 4
+    for (int r = warp; r < nr; r += kWarps)
+      for (int i = lane; i < run; i += 32) tile[r * pitch + i] = __ldg(from + r * nb * S + i);
+    __syncthreads();
+    int64_t* to = dst + ((win * N + t0) * R + r0) * S;
+    for (int t = warp; t < steps; t += kWarps) {
+      int r = lane / S, s = lane - r * S;
+#pragma unroll 4
+      for (int i = lane; i < nr * S; i += 32) {
+        to[t * R * S + i] = tile[r * pitch + t * S + s];
+        r += step_r;
+        s += step_s;
+        if (s >= S) {
+          s -= S;
+          ++r;
+        }
+      }
+    }
+    __syncthreads();
+  }
+}
+
 }  // namespace
 
 cudaError_t launch_gathered_to_steps(const int64_t* src, int64_t T, int64_t R, int64_t S, int64_t N, int64_t* dst,
                                      cudaStream_t stream) {
+  N = std::min(N, T);  // one window holds them all
+  if (use_tiles(R, S, N)) {
+    const int ranks = static_cast<int>(std::min<int64_t>(R, kTileBytes / (8 * tile_pitch(static_cast<int>(S)))));
+    const int64_t tiles = (T + N - 1) / N * ((N + kTileSteps - 1) / kTileSteps) * ((R + ranks - 1) / ranks);
+    const int grid = static_cast<int>(std::min<int64_t>(tiles, int64_t(sm_count()) * 4));
+    count_launch();
+    gathered_tiles_kernel<<<grid, kIngThreads, 0, stream>>>(src, T, R, static_cast<int>(S), N, ranks, dst);
+    return cudaGetLastError();
+  }
   const int unit = S % 2 == 0 ? 2 : 1;
   const int grid = static_cast<int>(std::min<int64_t>(T, int64_t(sm_count()) * 8));
   count_launch();

@@ -193,3 +193,16 @@ def test_group_lanes(sf, T, R, S, G, kind):
     g = sf.sf_group_aggregate(dev(d_np), dev(group), G, 100, t0=3, status=st)
     assert int(st.item()) == 0
     assert np.array_equal(host(g.X), np.transpose(o.X, (1, 0, 2))) and np.array_equal(host(g.D), o.D.T)
+
+
+# small steps: windows of a tile's 16 steps and one less and more, a short last
+# window, a tile of ranks and one more, the largest small step and the next
+@pytest.mark.parametrize("T,R,S,N", [(100, 16, 8, 16), (95, 31, 7, 15), (100, 47, 8, 17), (1000, 48, 8, 100),
+                                     (77, 49, 8, 40), (333, 383, 1, 50), (200, 385, 1, 64), (64, 12, 32, 33),
+                                     (40, 3, 3, 40), (19, 1, 1, 16), (30, 5, 4, 1 << 40)])
+def test_gathered_tiles(sf, T, R, S, N):
+    d = np.random.default_rng(T + R).integers(0, 1 << 62, size=(T, R, S), dtype=np.int64)
+    g = np.concatenate([d[t:t + N].transpose(1, 0, 2).reshape(-1) for t in range(0, T, N)])
+    out = torch.empty((T, R, S), dtype=torch.int64, device="cuda")
+    sf.sf_gathered_to_steps(dev(g), T, R, S, N, dst=out)
+    assert np.array_equal(host(out), d)
