@@ -16,7 +16,7 @@
 // warp group per step, spread over one or more tiles, with up to four groups
 // taking steps in turn (each group owning its ring stages).  The frontier over
 // steps of up to 6 KB takes 2-8 steps per warp instruction (lanes_kernel: groups
-// of lanes, one step each).  Fewer steps than SMs over many ranks split each
+// of lanes, one step each).  A few hundred steps over many ranks split each
 // step's ranks over a thread-block cluster (split_frontier_kernel).
 //
 // Generic path (17 to 32 stages; medians that are only 8-byte aligned): plain
@@ -38,28 +38,42 @@ namespace {
 
 template <int S>
 __device__ __forceinline__ void load_global_row(const int64_t* src, int64_t (&v)[S]) {
+  if constexpr (S % 2 == 0) {
 #pragma unroll
-  for (int j = 0; j < S / 2; ++j) {
-    const longlong2 x = __ldg(reinterpret_cast<const longlong2*>(src) + j);
-    v[2 * j] = x.x;
-    v[2 * j + 1] = x.y;
+    for (int j = 0; j < S / 2; ++j) {
+      const longlong2 x = __ldg(reinterpret_cast<const longlong2*>(src) + j);
+      v[2 * j] = x.x;
+      v[2 * j + 1] = x.y;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < S; ++j) v[j] = __ldg(src + j);
   }
 }
 
 // --------------------------------------------------------------------------
-// Few steps over many ranks (fewer steps than SMs: one window of a few
-// hundred steps, the per-window use of Sec. 3): each step's ranks are split
-// over a thread-block cluster of `csize` CTAs, so every SM streams.  CTA j of
-// the cluster reads ranks [j R / csize, (j+1) R / csize) with 16-byte loads
-// (four rows in flight per thread), reduces its packed per-stage keys
+// Few steps over many ranks (up to a few hundred steps of large jobs, the
+// per-window use of Sec. 3): each step's ranks are split over a thread-block
+// cluster of `csize` CTAs, all of them resident at once, so every SM streams and
+// no SM owns a whole step more than the others.  CTA j of the cluster reads ranks
+// [j R / csize, (j+1) R / csize) with 16-byte loads (8-byte ones for odd stage
+// counts; U rows in flight per thread), reduces its packed per-stage keys
 // (F << 16 | 65535 - r) to shared memory, and the cluster's first CTA takes
 // the maximum over the cluster's keys through distributed shared memory
 // (ranks are disjoint, so the largest key still carries the lowest attaining
 // rank) and runs the step's epilogue.  No global scratch.
+//
+// Two rows in flight per thread hold half the registers of four, so that half as
+// many CTAs again are resident and steps split further: frontier, us, four rows /
+// two: 100 x 8192 x 8 14.4 / 12.4, 160 x 8192 x 8 22.5 / 18.4, 200 x 32768 x 8
+// 72.7 / 65.9.  Where four rows split a step as well and leave a CTA 8192 ranks or
+// more, they are as fast or faster (64 x 65536 x 8 44.8 / 47.4, 140 x 16384 x 8
+// 27.3 / 28.4).
 constexpr int kSplitThreads = 256;
+constexpr int64_t kSplitLongShare = 8192;  // ranks of a CTA from which four rows are in flight
 constexpr int kSplitMaxCluster = 16;  // above 8: a non-portable cluster size, allowed per kernel
 
-template <int S>
+template <int S, int U>
 __global__ void __launch_bounds__(kSplitThreads) split_frontier_kernel(const int64_t* __restrict__ d, const Params p) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
@@ -75,7 +89,6 @@ __global__ void __launch_bounds__(kSplitThreads) split_frontier_kernel(const int
   FrontierRows<S> fr;
   fr.init();
   uint32_t dor = 0, tor = 0;
-  constexpr int U = 4;
   for (int64_t r = r0 + threadIdx.x; r < r1; r += int64_t(kSplitThreads) * U) {
     int64_t v[U][S];
 #pragma unroll
@@ -114,11 +127,11 @@ __global__ void __launch_bounds__(kSplitThreads) split_frontier_kernel(const int
   if (lane == 0) report(p.status, bits);
 }
 
-template <int S>
+template <int S, int U>
 cudaError_t launch_split(const int64_t* d, const Params& p, int csize, cudaStream_t stream, bool pdl) {
   static bool ready = false;  // attribute set once per process (same on every GB300)
   if (!ready) {
-    const cudaError_t e = cudaFuncSetAttribute(split_frontier_kernel<S>,
+    const cudaError_t e = cudaFuncSetAttribute(split_frontier_kernel<S, U>,
                                                cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     ready = true;
@@ -136,21 +149,21 @@ cudaError_t launch_split(const int64_t* d, const Params& p, int csize, cudaStrea
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, split_frontier_kernel<S>, d, p);
+  return cudaLaunchKernelEx(&cfg, split_frontier_kernel<S, U>, d, p);
 }
 
 // Cluster size for T steps over R ranks: the largest size (<= 16, at least
-// 512 ranks per CTA) at which all T clusters are resident at once.  A
+// 512 ranks per CTA) at which all T clusters are resident at once, 0 if none.  A
 // cluster is placed within one GPC, so sizes that do not divide a GPC's CTA
 // slots evenly fit fewer clusters than the SM count suggests, and a second
 // wave of clusters costs more than the parallelism gained (100 steps x 8192
 // ranks: 1, 3, 6 and 12 CTAs per step ran at 20.6, 21.9, 25.0 and 28.3 us).
 // The resident counts come from the occupancy calculator, once per process.
-template <int S>
+template <int S, int U>
 int split_cluster_size(int64_t T, int64_t R) {
   static const std::array<int, kSplitMaxCluster + 1> fit = [] {
     std::array<int, kSplitMaxCluster + 1> f{};
-    if (cudaFuncSetAttribute(split_frontier_kernel<S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+    if (cudaFuncSetAttribute(split_frontier_kernel<S, U>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
         cudaSuccess) {
       cudaGetLastError();
       return f;
@@ -167,7 +180,7 @@ int split_cluster_size(int64_t T, int64_t R) {
       cfg.attrs = attr;
       cfg.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, split_frontier_kernel<S>, &cfg) != cudaSuccess) {
+      if (cudaOccupancyMaxActiveClusters(&n, split_frontier_kernel<S, U>, &cfg) != cudaSuccess) {
         cudaGetLastError();
         n = 0;
       }
@@ -175,38 +188,75 @@ int split_cluster_size(int64_t T, int64_t R) {
     }
     return f;
   }();
-  int best = 1;
+  int best = fit[1] >= T ? 1 : 0;
   for (int c = 2; c <= kSplitMaxCluster; ++c)
     if (R / c >= 512 && fit[c] >= T) best = c;
   return best;
 }
 
+template <int U>
 int split_cluster(int S, int64_t T, int64_t R) {
   switch (S) {
-    case 2: return split_cluster_size<2>(T, R);
-    case 4: return split_cluster_size<4>(T, R);
-    case 6: return split_cluster_size<6>(T, R);
-    case 8: return split_cluster_size<8>(T, R);
-    case 10: return split_cluster_size<10>(T, R);
-    case 12: return split_cluster_size<12>(T, R);
-    case 14: return split_cluster_size<14>(T, R);
-    case 16: return split_cluster_size<16>(T, R);
-    default: return 1;
+    case 2: return split_cluster_size<2, U>(T, R);
+    case 3: return split_cluster_size<3, U>(T, R);
+    case 4: return split_cluster_size<4, U>(T, R);
+    case 5: return split_cluster_size<5, U>(T, R);
+    case 6: return split_cluster_size<6, U>(T, R);
+    case 7: return split_cluster_size<7, U>(T, R);
+    case 8: return split_cluster_size<8, U>(T, R);
+    case 9: return split_cluster_size<9, U>(T, R);
+    case 10: return split_cluster_size<10, U>(T, R);
+    case 11: return split_cluster_size<11, U>(T, R);
+    case 12: return split_cluster_size<12, U>(T, R);
+    case 14: return split_cluster_size<14, U>(T, R);
+    case 16: return split_cluster_size<16, U>(T, R);
+    default: return 0;
   }
 }
 
+template <int U>
 cudaError_t dispatch_split(int S, const int64_t* d, const Params& p, int csize, cudaStream_t stream, bool pdl) {
   switch (S) {
-    case 2: return launch_split<2>(d, p, csize, stream, pdl);
-    case 4: return launch_split<4>(d, p, csize, stream, pdl);
-    case 6: return launch_split<6>(d, p, csize, stream, pdl);
-    case 8: return launch_split<8>(d, p, csize, stream, pdl);
-    case 10: return launch_split<10>(d, p, csize, stream, pdl);
-    case 12: return launch_split<12>(d, p, csize, stream, pdl);
-    case 14: return launch_split<14>(d, p, csize, stream, pdl);
-    case 16: return launch_split<16>(d, p, csize, stream, pdl);
+    case 2: return launch_split<2, U>(d, p, csize, stream, pdl);
+    case 3: return launch_split<3, U>(d, p, csize, stream, pdl);
+    case 4: return launch_split<4, U>(d, p, csize, stream, pdl);
+    case 5: return launch_split<5, U>(d, p, csize, stream, pdl);
+    case 6: return launch_split<6, U>(d, p, csize, stream, pdl);
+    case 7: return launch_split<7, U>(d, p, csize, stream, pdl);
+    case 8: return launch_split<8, U>(d, p, csize, stream, pdl);
+    case 9: return launch_split<9, U>(d, p, csize, stream, pdl);
+    case 10: return launch_split<10, U>(d, p, csize, stream, pdl);
+    case 11: return launch_split<11, U>(d, p, csize, stream, pdl);
+    case 12: return launch_split<12, U>(d, p, csize, stream, pdl);
+    case 14: return launch_split<14, U>(d, p, csize, stream, pdl);
+    case 16: return launch_split<16, U>(d, p, csize, stream, pdl);
     default: return cudaErrorInvalidValue;
   }
+}
+
+// Whether a pass is split, and how: cluster size and rows in flight.  Any T that
+// is resident at once up to 12 stages (us, tiles / split: 160 x 8192 x 8 26.7 / 18.4,
+// 360 x 5965 x 8 36.8 / 28.9, 200 x 12345 x 6 36.8 / 22.8, 400 x 4001 x 4 16.6 / 10.4,
+// 300 x 5000 x 12 31.9 / 28.0, 200 x 5001 x 5 16.6 / 10.3, 360 x 5965 x 7 32.8 / 26.7,
+// 100 x 8001 x 7 18.5 / 10.4); with more, whose rows of 128 bytes a lane the loads
+// serve badly, only fewer steps than SMs (300 x 4000 x 16 33.0 / 39.0,
+// 160 x 16384 x 16 82 / 134).
+struct Split {
+  int csize = 0;
+  int rows = 0;
+};
+
+Split plan_split(const StreamJob& j, int sms) {
+  Split q;
+  if (j.gain || j.base || j.R < 1024 || j.S > 16 || (j.S > 12 && j.T >= sms) || j.T > int64_t(sms) * 8) return q;
+  if (j.S % 2 == 0 && reinterpret_cast<uintptr_t>(j.d) % 16 != 0) return q;
+  const int S = static_cast<int>(j.S);
+  q.rows = 4;
+  q.csize = split_cluster<4>(S, j.T, j.R);
+  if (q.csize > 1 && j.R / q.csize >= kSplitLongShare) return q;
+  q.rows = 2;
+  q.csize = split_cluster<2>(S, j.T, j.R);
+  return q;
 }
 
 // --------------------------------------------------------------------------
@@ -566,16 +616,19 @@ cudaError_t launch_stream_pass(const StreamJob& j, cudaStream_t stream) {
   const bool fast = j.S <= 16 && rows >= 1 && rows <= int64_t(0x7fffffff) && encode_fn() != nullptr &&
                     (!j.gain || reinterpret_cast<uintptr_t>(j.m) % 16 == 0);
   const int sms = sm_count();
-  // fewer steps than SMs over many ranks (frontier and aggregation): split
-  // each step's ranks over a cluster so that every SM streams
-  if (!j.gain && !j.base && j.T < sms && j.R >= 1024 && (j.S % 2 == 0) && j.S <= 16 &&
-      reinterpret_cast<uintptr_t>(j.d) % 16 == 0) {
-    const int csize = split_cluster(static_cast<int>(j.S), j.T, j.R);
+  // few steps over many ranks (frontier and aggregation): split each step's
+  // ranks over a cluster so that every SM streams
+  if (const Split q = plan_split(j, sms); q.csize > 0) {
+    auto go = [&](int csize) {
+      const int S = static_cast<int>(j.S);
+      return q.rows == 4 ? dispatch_split<4>(S, j.d, p, csize, stream, j.after_clear)
+                         : dispatch_split<2>(S, j.d, p, csize, stream, j.after_clear);
+    };
     count_launch();
-    cudaError_t e = dispatch_split(static_cast<int>(j.S), j.d, p, csize, stream, j.after_clear);
-    if (e != cudaSuccess && csize > 8) {  // a 16-CTA cluster that cannot be placed: portable size
+    cudaError_t e = go(q.csize);
+    if (e != cudaSuccess && q.csize > 8) {  // a 16-CTA cluster that cannot be placed: portable size
       cudaGetLastError();
-      e = dispatch_split(static_cast<int>(j.S), j.d, p, 8, stream, j.after_clear);
+      e = go(8);
     }
     return e;
   }

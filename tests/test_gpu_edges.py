@@ -206,3 +206,23 @@ def test_gathered_tiles(sf, T, R, S, N):
     out = torch.empty((T, R, S), dtype=torch.int64, device="cuda")
     sf.sf_gathered_to_steps(dev(g), T, R, S, N, dst=out)
     assert np.array_equal(host(out), d)
+
+
+# few steps of many ranks: odd stage counts, T at the SM count, at the most that are
+# resident at once and past it, whole clusters and single CTAs per step, shares of
+# 8192 ranks and more (four rows in flight), the fewest ranks and one less
+@pytest.mark.parametrize("T,R,S", [(3, 1025, 3), (100, 5001, 5), (305, 1100, 7), (2, 9000, 9), (40, 1500, 11),
+                                   (151, 1024, 8), (152, 1023, 8), (153, 1025, 8), (456, 1100, 8), (457, 1100, 8),
+                                   (762, 1030, 4), (160, 2100, 10), (60, 16500, 12), (151, 2000, 14), (152, 2000, 14),
+                                   (200, 1030, 13), (900, 1024, 2)])
+@pytest.mark.parametrize("kind", ["ms", "long"])
+def test_split_steps(sf, T, R, S, kind):
+    d_np = durations(T, R, S, kind, T + R + S)
+    d, st = dev(d_np), sf.new_status("cuda")
+    f, o = sf.sf_frontier(d, status=st), O.frontier(d_np)
+    assert np.array_equal(host(f.a), o.a) and np.array_equal(host(f.lead), o.lead)
+    assert np.array_equal(host(f.makespan), o.makespan)
+    win, ow = sf.sf_window_aggregate(d, 50, t0=7, status=st), O.windows(d_np, 50, 7)
+    assert np.array_equal(host(win.X), ow.X) and np.array_equal(host(win.E), ow.E)
+    assert np.array_equal(host(win.C), ow.C) and np.array_equal(host(win.step_lead), ow.step_lead)
+    assert int(st.item()) == 0
