@@ -23,6 +23,8 @@
 #include <cstdint>
 #include <type_traits>
 
+#include <cooperative_groups.h>
+
 #include "sf_device.cuh"
 #include "sf_lane_select.cuh"
 #include "sf_launch.h"
@@ -99,10 +101,28 @@ __device__ __forceinline__ void fold_row(const GroupParams& p, const int64_t* ro
   tor |= static_cast<uint32_t>(static_cast<uint64_t>(P) >> 32);
 }
 
+// Entry i of the step's F_g: the CTA's own, or the largest over the cluster's CTAs.
+template <bool SPLIT>
+__device__ __forceinline__ int64_t step_frontier(unsigned long long* Fk, int i, int csize, int rank) {
+  unsigned long long F = Fk[i];
+  if constexpr (SPLIT) {
+    for (int c = 1; c < csize; ++c) {
+      const int other = rank + c < csize ? rank + c : rank + c - csize;
+      const unsigned long long x =
+          *cooperative_groups::this_cluster().map_shared_rank(&Fk[i], static_cast<unsigned>(other));
+      F = x > F ? x : F;
+    }
+  }
+  return static_cast<int64_t>(F);
+}
+
 // Dynamic shared memory: Fk [G][S] u64 (this step's group frontier),
-// accX [G][S] i64 and accD [G] i64 (the current window's sums).
-template <int SC>
+// accX [G][S] i64 and accD [G] i64 (the current window's sums).  SPLIT: a cluster
+// of CTAs shares each step's ranks, and its CTAs combine their Fk through
+// distributed shared memory, each for every csize-th group.
+template <int SC, bool SPLIT>
 __global__ void __launch_bounds__(kGrThreads) group_window_kernel(const GroupParams p) {
+  namespace cg = cooperative_groups;
   extern __shared__ __align__(16) unsigned char dyn[];
   const int S = SC > 0 ? SC : static_cast<int>(p.S);
   const int G = static_cast<int>(p.G), GS = G * S;
@@ -111,7 +131,15 @@ __global__ void __launch_bounds__(kGrThreads) group_window_kernel(const GroupPar
   int64_t* accD = accX + GS;
   const int tid = threadIdx.x, lane = tid & 31;
   const int64_t R = p.R;
-  const int64_t nb = gridDim.x, b = blockIdx.x;
+  int csize = 1, rank = 0;
+  if constexpr (SPLIT) {
+    csize = static_cast<int>(cg::this_cluster().num_blocks());
+    rank = static_cast<int>(cg::this_cluster().block_rank());
+  }
+  // the CTA's ranks: whole warps, so that a warp's ranks stay those of a node
+  const int64_t r_begin = SPLIT ? (R + 31) / 32 * rank / csize * 32 : 0;
+  const int64_t r_end = SPLIT ? min(R, (R + 31) / 32 * (rank + 1) / csize * 32) : R;
+  const int64_t nb = gridDim.x / csize, b = blockIdx.x / csize;
   const int64_t q = p.T / nb, rr = p.T % nb;
   const int64_t t_begin = q * b + (b < rr ? b : rr), t_end = t_begin + q + (b < rr ? 1 : 0);
   uint32_t dor = 0, tor = 0, bad_group = 0;
@@ -143,12 +171,12 @@ __global__ void __launch_bounds__(kGrThreads) group_window_kernel(const GroupPar
     __syncthreads();
     const int64_t* dt = p.d + t * R * S;
     constexpr int kRows = (SC > 0 && SC <= 8) ? 2 : 1;
-    for (int64_t base = tid - lane; base < R; base += int64_t(kRows) * kGrThreads) {
+    for (int64_t base = r_begin + tid - lane; base < r_end; base += int64_t(kRows) * kGrThreads) {
       // warp-uniform loop: every lane takes part in the warp reductions
 #pragma unroll
       for (int k = 0; k < kRows; ++k) {
         const int64_t r = base + int64_t(k) * kGrThreads + lane;
-        const bool in = r < R;
+        const bool in = r < r_end;
         int g = in ? __ldg(p.group + r) : -1;
         const bool ok = g >= 0 && g < G;
         bad_group |= (in && !ok) ? 1u : 0u;
@@ -158,15 +186,24 @@ __global__ void __launch_bounds__(kGrThreads) group_window_kernel(const GroupPar
         fold_row<SC>(p, dt + (in ? r : 0) * S, S, g, ok, uniform, Fk, dor, tor);
       }
     }
-    __syncthreads();
+    if constexpr (SPLIT) {
+      cg::this_cluster().sync();
+    } else {
+      __syncthreads();
+    }
     // the step's group increments a_g[s] = F_g[s] - F_g[s-1] and makespans
     for (int i = tid; i < GS; i += kGrThreads) {
       const int s = i % S;
-      const int64_t F = static_cast<int64_t>(Fk[i]);
-      accX[i] += F - (s > 0 ? static_cast<int64_t>(Fk[i - 1]) : 0);
+      if (SPLIT && i / S % csize != rank) continue;
+      const int64_t F = step_frontier<SPLIT>(Fk, i, csize, rank);
+      accX[i] += F - (s > 0 ? step_frontier<SPLIT>(Fk, i - 1, csize, rank) : 0);
       if (s == S - 1) accD[i / S] += F;
     }
-    __syncthreads();
+    if constexpr (SPLIT) {
+      cg::this_cluster().sync();  // the others read Fk until here
+    } else {
+      __syncthreads();
+    }
   }
   if (cur_w >= 0) {
     for (int i = tid; i < GS; i += kGrThreads)
@@ -344,7 +381,7 @@ __global__ void stage_group_sum_kernel(const int64_t* __restrict__ X, int64_t nW
 
 template <int SC>
 cudaError_t launch_group_t(const GroupParams& p, size_t smem, cudaStream_t stream) {
-  auto kern = group_window_kernel<SC>;
+  auto kern = group_window_kernel<SC, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   int per_sm = 0;
@@ -352,9 +389,32 @@ cudaError_t launch_group_t(const GroupParams& p, size_t smem, cudaStream_t strea
     cudaGetLastError();
     per_sm = 1;
   }
-  const int grid = static_cast<int>(std::min<int64_t>(int64_t(per_sm) * sm_count(), p.T));
+  const int64_t slots = int64_t(per_sm) * sm_count();
   count_launch();
-  kern<<<grid, kGrThreads, smem, stream>>>(p);
+  // few steps of many ranks: CTAs enough for every SM, at least 1024 ranks each (us, a
+  // CTA per step / split: 1 x 8192 x 8 47 / 16, 100 x 8192 x 8 49 / 25, 250 x 8192 x 8
+  // 62 / 41, 100 x 30000 x 16 299 / 130; two CTAs for 1024 ranks, 300 x 1024 x 6 12 / 14)
+  int csize = 1;
+  while (csize < 8 && p.T * csize * 2 <= slots && p.R >= int64_t(csize) * 2048) csize *= 2;
+  if (csize > 1) {
+    auto split = group_window_kernel<SC, true>;
+    e = cudaFuncSetAttribute(split, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(csize);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(static_cast<unsigned>(p.T * csize));
+    cfg.blockDim = dim3(kGrThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, split, p);
+  }
+  kern<<<static_cast<unsigned>(std::min(slots, p.T)), kGrThreads, smem, stream>>>(p);
   return cudaGetLastError();
 }
 

@@ -226,3 +226,19 @@ def test_split_steps(sf, T, R, S, kind):
     assert np.array_equal(host(win.X), ow.X) and np.array_equal(host(win.E), ow.E)
     assert np.array_equal(host(win.C), ow.C) and np.array_equal(host(win.step_lead), ow.step_lead)
     assert int(st.item()) == 0
+
+
+# few steps: a step's ranks over a cluster of two, four and eight CTAs, in shares that
+# end inside a group, groups in blocks and mixed
+@pytest.mark.parametrize("T,R,S,G", [(1, 8191, 8, 64), (90, 8200, 6, 61), (150, 4097, 10, 33), (300, 2048, 4, 300),
+                                     (20, 17000, 18, 130), (200, 2049, 16, 9), (7, 30001, 3, 3)])
+@pytest.mark.parametrize("kind", ["blocks", "mixed", "long"])
+def test_few_steps_groups(sf, T, R, S, G, kind):
+    d_np = durations(T, R, S, "long" if kind == "long" else "ms", T + R)
+    group = np.random.default_rng(T).integers(0, G, size=R)
+    group = (group if kind == "mixed" else np.sort(group)).astype(np.int32)
+    o = O.group_windows(d_np, group, G, 40, 3)
+    st = sf.new_status("cuda")
+    g = sf.sf_group_aggregate(dev(d_np), dev(group), G, 40, t0=3, status=st)
+    assert int(st.item()) == 0
+    assert np.array_equal(host(g.X), np.transpose(o.X, (1, 0, 2))) and np.array_equal(host(g.D), o.D.T)
