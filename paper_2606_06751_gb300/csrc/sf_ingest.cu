@@ -17,19 +17,32 @@ constexpr int kIngThreads = 256;
 
 // dst[t][r][s] = src block b = t / N, [r][t - b*N][s]; block b starts at
 // element b*R*N*S and holds n_b = min(N, T - b*N) steps.  A CTA fills one
-// destination step at a time.
-template <int kUnit>  // int64 values moved per thread: 2 (S even) or 1
+// destination step at a time, with PARTS one of `parts` pieces of a step: few
+// steps of many ranks then have eight CTAs per SM (us: 1 x 8192 x 8 19.4 -> 6.3,
+// 100 x 8192 x 8 51 -> 20, 250 x 8192 x 8 66 -> 46, 100 x 30000 x 16 347 -> 129).
+// The piece's arithmetic slows small steps (100000 x 128 x 8 263 -> 401).
+template <int kUnit, bool PARTS>  // kUnit int64 values moved per thread: 2 (S even) or 1
 __global__ void __launch_bounds__(kIngThreads) gathered_to_steps_kernel(const int64_t* __restrict__ src, int64_t T,
                                                                         int64_t R, int64_t S, int64_t N,
-                                                                        int64_t* __restrict__ dst) {
+                                                                        int parts, int64_t* __restrict__ dst) {
   const int units = static_cast<int>(R * S / kUnit);  // per destination step (<= 2^21)
   const int su = static_cast<int>(S / kUnit);
-  for (int64_t t = blockIdx.x; t < T; t += gridDim.x) {
+  const int64_t pieces = PARTS ? T * parts : T;
+  for (int64_t id = blockIdx.x; id < pieces; id += gridDim.x) {
+    int64_t t = id;
+    int begin = 0, end = units;
+    if constexpr (PARTS) {
+      t = id / parts;
+      const int part = static_cast<int>(id - t * parts);
+      begin = static_cast<int>(int64_t(units) * part / parts);
+      end = static_cast<int>(int64_t(units) * (part + 1) / parts);
+    }
     const int64_t b = t / N, tl = t - b * N;
     const int64_t nb = T - b * N < N ? T - b * N : N;
     const int64_t* sb = src + b * R * N * S + tl * S;
     int64_t* dt = dst + t * R * S;
-    for (int j = threadIdx.x; j < units; j += kIngThreads) {
+#pragma unroll 4
+    for (int j = begin + threadIdx.x; j < end; j += kIngThreads) {
       const int r = j / su;
       const int s = (j - r * su) * kUnit;
       const int64_t* from = sb + int64_t(r) * nb * S + s;
@@ -113,12 +126,13 @@ cudaError_t launch_gathered_to_steps(const int64_t* src, int64_t T, int64_t R, i
     return cudaGetLastError();
   }
   const int unit = S % 2 == 0 ? 2 : 1;
-  const int grid = static_cast<int>(std::min<int64_t>(T, int64_t(sm_count()) * 8));
+  const int64_t slots = int64_t(sm_count()) * 8;
+  const int parts = static_cast<int>(std::min(slots / T, R * S / (4096 * unit)));  // at least 4096 units each
+  const int grid = static_cast<int>(std::min(T * std::max(parts, 1), slots));
   count_launch();
-  if (unit == 2)
-    gathered_to_steps_kernel<2><<<grid, kIngThreads, 0, stream>>>(src, T, R, S, N, dst);
-  else
-    gathered_to_steps_kernel<1><<<grid, kIngThreads, 0, stream>>>(src, T, R, S, N, dst);
+  auto go = [&](auto kern) { kern<<<grid, kIngThreads, 0, stream>>>(src, T, R, S, N, parts, dst); };
+  if (unit == 2) parts > 1 ? go(gathered_to_steps_kernel<2, true>) : go(gathered_to_steps_kernel<2, false>);
+  else parts > 1 ? go(gathered_to_steps_kernel<1, true>) : go(gathered_to_steps_kernel<1, false>);
   return cudaGetLastError();
 }
 

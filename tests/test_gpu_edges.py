@@ -242,3 +242,15 @@ def test_few_steps_groups(sf, T, R, S, G, kind):
     g = sf.sf_group_aggregate(dev(d_np), dev(group), G, 40, t0=3, status=st)
     assert int(st.item()) == 0
     assert np.array_equal(host(g.X), np.transpose(o.X, (1, 0, 2))) and np.array_equal(host(g.D), o.D.T)
+
+
+# few steps of many ranks, moved in pieces: whole and ragged ones, odd and even stage
+# counts, the fewest units that are split and one rank less, a short last window
+@pytest.mark.parametrize("T,R,S,N", [(1, 8191, 8, 1), (90, 8200, 6, 40), (7, 30001, 3, 2), (400, 2048, 8, 150),
+                                     (400, 2047, 8, 150), (20, 2731, 3, 7), (20, 2730, 3, 7)])
+def test_gathered_pieces(sf, T, R, S, N):
+    d = np.random.default_rng(T + R).integers(0, 1 << 62, size=(T, R, S), dtype=np.int64)
+    g = np.concatenate([d[t:t + N].transpose(1, 0, 2).reshape(-1) for t in range(0, T, N)])
+    out = torch.empty((T, R, S), dtype=torch.int64, device="cuda")
+    sf.sf_gathered_to_steps(dev(g), T, R, S, N, dst=out)
+    assert np.array_equal(host(out), d)
