@@ -48,8 +48,8 @@ METRIC = "rank·step·stage records/sec and achieved HBM GB/s (% of GB300 peak)"
 UNIT = "records/s"
 # the sources each roofline kernel is compiled from: a recorded DRAM traffic
 # figure is valid only while their hash is the one it was captured with
-KERNEL_SOURCES = {"window_median": ("sf_select.cu", "sf_device.cuh"),
-                  "direct_gain": ("sf_stream.cu", "sf_device.cuh")}
+KERNEL_SOURCES = {"window_median": ("sf_select.cu", "sf_lane_select.cuh", "sf_warp_select.cuh", "sf_device.cuh"),
+                  "direct_gain": ("sf_stream.cu", "sf_stream.cuh", "sf_tiled.cuh", "sf_device.cuh")}
 
 
 # --------------------------------------------------------------------------- distributed harness
