@@ -445,14 +445,28 @@ cudaError_t launch_group_windows(const int64_t* d, int64_t T, int64_t R, int64_t
     return launch_group_lanes<5>(p, stream);
   }
   const size_t smem = size_t(G) * S * 16 + size_t(G) * 8;
+  // Stage counts known to the compiler, whose rows are loaded ahead of their reductions
+  // (us, loop over the stages / unrolled: 13421 x 1000 x 5 139 / 115, 10000 x 1024 x 9
+  // 184 / 139, 10000 x 700 x 11 174 / 133; 8000 x 1000 x 14 199 / 204).  Up to eight stages
+  // a warp takes two rows of 256 ranks, one of them idle in smaller steps (60000 x 200 x 7
+  // 233 / 268).
+  const bool two_rows = R > kGrThreads;
   switch (S) {
+    case 2: if (two_rows) return launch_group_t<2>(p, smem, stream); break;
+    case 3: if (two_rows) return launch_group_t<3>(p, smem, stream); break;
+    case 5: if (two_rows) return launch_group_t<5>(p, smem, stream); break;
+    case 7: if (two_rows) return launch_group_t<7>(p, smem, stream); break;
     case 4: return launch_group_t<4>(p, smem, stream);
     case 6: return launch_group_t<6>(p, smem, stream);
     case 8: return launch_group_t<8>(p, smem, stream);
+    case 9: return launch_group_t<9>(p, smem, stream);
     case 10: return launch_group_t<10>(p, smem, stream);
+    case 11: return launch_group_t<11>(p, smem, stream);
+    case 12: return launch_group_t<12>(p, smem, stream);
     case 16: return launch_group_t<16>(p, smem, stream);
-    default: return launch_group_t<0>(p, smem, stream);
+    default: break;
   }
+  return launch_group_t<0>(p, smem, stream);
 }
 
 cudaError_t launch_stage_group_sum(const int64_t* X, int64_t nW, int64_t S, const int32_t* stage_group, int64_t K,

@@ -20,7 +20,7 @@ constexpr int kIngThreads = 256;
 // destination step at a time, with PARTS one of `parts` pieces of a step: few
 // steps of many ranks then have eight CTAs per SM (us: 1 x 8192 x 8 19.4 -> 6.3,
 // 100 x 8192 x 8 51 -> 20, 250 x 8192 x 8 66 -> 46, 100 x 30000 x 16 347 -> 129).
-// The piece's arithmetic slows small steps (100000 x 128 x 8 263 -> 401).
+// One kernel for both forms read slower over many steps (100000 x 128 x 8 263 -> 401).
 template <int kUnit, bool PARTS>  // kUnit int64 values moved per thread: 2 (S even) or 1
 __global__ void __launch_bounds__(kIngThreads) gathered_to_steps_kernel(const int64_t* __restrict__ src, int64_t T,
                                                                         int64_t R, int64_t S, int64_t N,

@@ -228,6 +228,19 @@ def test_split_steps(sf, T, R, S, kind):
     assert int(st.item()) == 0
 
 
+# every stage count of its own kernel and those without, in steps of one and two
+# rows of 256 ranks, more groups than the lanes take
+@pytest.mark.parametrize("T,R,S", [(500, r, s) for s in (2, 3, 5, 7, 9, 11, 12, 13) for r in (256, 257, 513)])
+def test_group_stages(sf, T, R, S):
+    d_np = durations(T, R, S, "ms", R + S)
+    group = np.sort(np.random.default_rng(S).integers(0, 33, size=R)).astype(np.int32)
+    o = O.group_windows(d_np, group, 33, 90, 3)
+    st = sf.new_status("cuda")
+    g = sf.sf_group_aggregate(dev(d_np), dev(group), 33, 90, t0=3, status=st)
+    assert int(st.item()) == 0
+    assert np.array_equal(host(g.X), np.transpose(o.X, (1, 0, 2))) and np.array_equal(host(g.D), o.D.T)
+
+
 # few steps: a step's ranks over a cluster of two, four and eight CTAs, in shares that
 # end inside a group, groups in blocks and mixed
 @pytest.mark.parametrize("T,R,S,G", [(1, 8191, 8, 64), (90, 8200, 6, 61), (150, 4097, 10, 33), (300, 2048, 4, 300),
