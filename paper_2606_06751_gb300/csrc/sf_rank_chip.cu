@@ -30,6 +30,7 @@
 // totals below 4.29 s) orders by them as they are; otherwise the step is read
 // again and keys are taken relative to rank 0's value, exact while no value is
 // 2^31 or more away from it; a step where one is selects on 64-bit values.
+#include "sf_bracket.h"
 #include "sf_rank_chip.cuh"
 #include "sf_warp_select.cuh"
 
@@ -369,28 +370,28 @@ __global__ void __launch_bounds__(kStepThreads, 2) rank_step_kernel(const ChipPa
           A = lo;
           B = k1;
         }
-        // the median is the rem-th key (from 0) of those in [A, B]
+        // the median is the rem-th key (from 0) of those in the bracket
+        KeyBracket br = KeyBracket::between(A, B);
         uint32_t rem = kth, ans = lo;
         bool first = true;
-        while (lo != k1) {
-          const uint32_t span = B - A;
-          const int bits = span ? 32 - __clz(static_cast<int>(span)) : 0, sh = bits > 8 ? bits - 8 : 0;
+        for (int round = 0; lo != k1 && round < kBracketRounds; ++round) {
+          const int sh = br.shift();
           for (int i = gl; i < 64; i += gn) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0, 0, 0, 0);
           if (gl == 0) *ncand = 0;
           group_sync();
           if (first) {
-            uint32_t out = 0;  // keys below A in the low half word, above B in the high one
+            uint32_t out = 0;  // keys below the bracket in the low half word, above it in the high one
             each([&](uint32_t x) {
-              const uint32_t o = x - A;
-              red_shared_inc_if(&hist[(o >> sh) & 255u], o <= span);
-              out += o <= span ? 0u : x < A ? 1u : 0x10000u;
+              const uint32_t o = x - br.lo;
+              red_shared_inc_if(&hist[(o >> sh) & 255u], o <= br.span);
+              out += o <= br.span ? 0u : x < br.lo ? 1u : 0x10000u;
             });
             out = __reduce_add_sync(kFull, out);
             if (lane == 0) part[40 + (gl >> 5)] = out;
           } else {
             each([&](uint32_t x) {
-              const uint32_t o = x - A;
-              red_shared_inc_if(&hist[(o >> sh) & 255u], o <= span);
+              const uint32_t o = x - br.lo;
+              red_shared_inc_if(&hist[(o >> sh) & 255u], o <= br.span);
             });
           }
           group_sync();
@@ -401,11 +402,9 @@ __global__ void __launch_bounds__(kStepThreads, 2) rank_step_kernel(const ChipPa
             const uint32_t below = out & 0xffffu, upto = static_cast<uint32_t>(R) - (out >> 16);
             if (kth < below || kth >= upto) {  // outside the bracket
               if (kth < below) {
-                B = A - 1;
-                A = lo;
+                br = KeyBracket::between(lo, br.lo - 1);
               } else {
-                A = B + 1;
-                B = k1;
+                br = KeyBracket::between(br.last() + 1, k1);
                 rem = kth - upto;
               }
               group_sync();  // every warp has read the counts
@@ -417,14 +416,12 @@ __global__ void __launch_bounds__(kStepThreads, 2) rank_step_kernel(const ChipPa
           hist_find(hist, rem, lane, digit, less);
           const uint32_t kept = hist[digit];
           rem -= less;
-          A += digit << sh;
-          B = min(B, A + ((1u << sh) - 1u));
-          ans = A;
+          br.narrow(digit);
+          ans = br.lo;
           if (sh == 0) break;
           if (kept <= 32) {
-            const uint32_t width = B - A;
             each([&](uint32_t x) {
-              if (x - A <= width) cbuf[atomicAdd(ncand, 1u) & 31u] = x;
+              if (br.has(x)) cbuf[atomicAdd(ncand, 1u) & 31u] = x;
             });
             group_sync();
             const uint32_t v = static_cast<uint32_t>(lane) < kept ? cbuf[lane] : 0xffffffffu;

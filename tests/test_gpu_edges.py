@@ -267,3 +267,26 @@ def test_gathered_pieces(sf, T, R, S, N):
     out = torch.empty((T, R, S), dtype=torch.int64, device="cuda")
     sf.sf_gathered_to_steps(dev(g), T, R, S, N, dst=out)
     assert np.array_equal(host(out), d)
+
+
+# columns in shared memory whose median lies in the last bins below 2^32, by their
+# values and relative to rank 0: one to eight warps per column
+@pytest.mark.parametrize("T,R,S", [(6, 4000, 3), (5, 2500, 6), (4, 9000, 2), (5, 2050, 11), (3, 11001, 1), (200, 3000, 4)])
+@pytest.mark.parametrize("relative", [False, True])
+@pytest.mark.parametrize("late", [1 << 23, 64])
+def test_rank_bracket_at_word_end(sf, T, R, S, relative, late):
+    rng = np.random.default_rng(T + R + S)
+    d_np = rng.integers(0, 8, size=(T, R, S))
+    top = (1 << 31 if relative else 1 << 32) - 8 * S - 1
+    waits = rng.random((T, R)) < 0.25
+    d_np[..., 0] = np.where(waits, rng.integers(top // 2, top * 3 // 4, size=(T, R)), top - rng.integers(late, size=(T, R)))
+    if relative:
+        d_np[:, 0, 0] = 0
+        d_np[..., 0] += 1 << 33
+    o = O.rank_lag(d_np)
+    st = sf.new_status("cuda")
+    g = sf.sf_rank_lag(dev(d_np), status=st)
+    sp = sf.sf_raw_spread(dev(d_np), 4, t0=3, status=st)
+    assert int(st.item()) == 0
+    assert np.array_equal(host(g.L), o.L) and np.array_equal(host(g.dL), o.dL) and np.array_equal(host(g.G), o.G)
+    assert np.array_equal(host(sp), O.raw_spread(d_np, 4, 3))
