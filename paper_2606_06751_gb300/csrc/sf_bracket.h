@@ -4,11 +4,7 @@
 
 #include <stdint.h>
 
-#ifdef __CUDACC__
-#define SF_HOST_DEVICE __host__ __device__ __forceinline__
-#else
-#define SF_HOST_DEVICE inline
-#endif
+#include "sf_host_device.h"
 
 namespace sf {
 

@@ -20,6 +20,7 @@
 // rows' stride already spreads them.
 #pragma once
 
+#include "sf_median_slots.h"
 #include "sf_stream.cuh"
 
 namespace sf {
@@ -109,31 +110,10 @@ struct GroupRing {
 };
 
 
-// Window slots of resident medians.  Window i of the CTA's range (0, 1, ...)
-// lives in slot i % slots.  Every consumer warp arrives on a window's `done`
-// barrier once, in order, when it is past the window (whether or not it had a
-// step in it) and before it waits for anything later; the producer refills a
-// slot when all have.
+// Window slots of resident medians (sf_median_slots.h) and their barriers.
 struct MedianSlots {
   unsigned char* base;
   uint64_t *full, *done;  // [2] each
-  __device__ __forceinline__ uint32_t slot(const Params& p, int i) const {
-    return p.m_slots == 2 ? static_cast<uint32_t>(i) & 1u : 0u;
-  }
-  __device__ __forceinline__ uint32_t parity(const Params& p, int i) const {
-    return static_cast<uint32_t>(p.m_slots == 2 ? i >> 1 : i) & 1u;
-  }
-};
-
-// A consumer warp's place among the windows.
-struct MedianWalk {
-  int at = -1;  // window the warp is in
-  __device__ __forceinline__ void pass_to(const Params& p, const MedianSlots& ms, int i, int lane) {
-    if (at >= i) return;
-    __syncwarp();  // every lane's reads of the windows left behind are done
-    for (; at < i; ++at)
-      if (at >= 0 && lane == 0) mbar_arrive(&ms.done[ms.slot(p, at)]);
-  }
 };
 
 // Producer q of kProducers (one thread each) issues the copies of the stages
@@ -169,13 +149,14 @@ __device__ void produce(int q, const CUtensorMap* map, const CUtensorMap* map_m,
   };
   WinTrack mw;  // window of the medians (evidence pass)
   int m_next = 0;  // windows of resident medians issued
+  const MedianPlace place{p.m_slots};
   const int64_t w_base = p.m_slots ? t_begin / p.W : 0;
   // producer 0: the resident medians of every window up to that of step t
   auto medians_to = [&](int64_t t) {
     if (q != 0 || !p.m_slots) return;
     for (const int last = static_cast<int>(mw.at(t, 0, p.W, 0) - w_base); m_next <= last && ok; ++m_next) {
-      const uint32_t sl = ms.slot(p, m_next);
-      if (!mbar_wait_bounded(&ms.done[sl], ms.parity(p, m_next) ^ 1u, abort)) {
+      const uint32_t sl = place.slot(m_next);
+      if (!mbar_wait_bounded(&ms.done[sl], place.parity(m_next) ^ 1u, abort)) {
         ok = false;
         return;
       }
@@ -216,7 +197,7 @@ __device__ void produce(int q, const CUtensorMap* map, const CUtensorMap* map_m,
   for (uint32_t st = 0; st < kMaxStages; ++st)
     if ((used >> st) & 1u) mbar_wait_timeout(&full[st], (last_ph >> st) & 1u);
   for (int i = max(0, m_next - p.m_slots); i < m_next; ++i)
-    mbar_wait_timeout(&ms.full[ms.slot(p, i)], ms.parity(p, i));
+    mbar_wait_timeout(&ms.full[place.slot(i)], place.parity(i));
 }
 
 // --------------------------------------------------------------------------
@@ -273,18 +254,22 @@ __global__ void __launch_bounds__((consumer_warps(KIND, S) + kProducers) * 32, 1
   const int64_t RS = p.R * S;
   // resident medians of a step's window: the slot, once they have landed
   [[maybe_unused]] MedianWalk mwalk;
+  [[maybe_unused]] const MedianPlace place{p.m_slots};
   [[maybe_unused]] const int64_t w_base = GAIN && p.m_slots ? t_begin / p.W : 0;
   [[maybe_unused]] bool m_have = true;
-  int m_in = -1;  // the window whose medians were waited for
+  auto hand_back = [&](int i) {
+    if (lane == 0) mbar_arrive(&ms.done[place.slot(i)]);
+  };
+  auto landed = [&](int i) {
+    if (!mbar_wait_bounded(&ms.full[place.slot(i)], place.parity(i), abort)) m_have = false;
+  };
   auto enter = [&](int64_t w) {
     const int i = static_cast<int>(w - w_base);
-    if (m_in == i) return;
-    m_in = i;
-    mwalk.pass_to(p, ms, i, lane);
-    const uint32_t sl = ms.slot(p, i);
-    m_have = mbar_wait_bounded(&ms.full[sl], ms.parity(p, i), abort);
+    if (mwalk.at == i) return;
+    __syncwarp();  // every lane's reads of the window left behind are done
+    mwalk.enter(i, hand_back, landed);
     if (!ALIGNED && m_have)
-      patch_tail<kSwz>(ms.base + size_t(sl) * p.m_bytes, p.m, p.m_rows, w * RS, static_cast<int>(RS), lane);
+      patch_tail<kSwz>(ms.base + size_t(place.slot(i)) * p.m_bytes, p.m, p.m_rows, w * RS, static_cast<int>(RS), lane);
   };
 
   if (p.regime == 0) {
@@ -482,7 +467,7 @@ __global__ void __launch_bounds__((consumer_warps(KIND, S) + kProducers) * 32, 1
               int64_t mfirst = w * RS + rank_tile0 * S;
               int mrank0 = rank_tile0;
               if (p.m_slots) {
-                mtile = ms.base + size_t(ms.slot(p, mwalk.at)) * p.m_bytes;
+                mtile = ms.base + size_t(place.slot(mwalk.at)) * p.m_bytes;
                 mfirst = w * RS;
                 mrank0 = 0;
               } else if constexpr (!ALIGNED) {
@@ -567,9 +552,12 @@ __global__ void __launch_bounds__((consumer_warps(KIND, S) + kProducers) * 32, 1
     else if (p.groups == 2) consume(std::integral_constant<int, 2>{});
     else consume(std::integral_constant<int, 1>{});
   }
-  // past every window: the producer may still wait for a slot that other warps need
+  // no more steps: the producer may still wait for a slot that other warps need
   if constexpr (GAIN)
-    if (p.m_slots && t_end > t_begin) mwalk.pass_to(p, ms, static_cast<int>((t_end - 1) / p.W - w_base) + 1, lane);
+    if (p.m_slots && t_end > t_begin) {
+      __syncwarp();
+      mwalk.leave(static_cast<int>((t_end - 1) / p.W - w_base), p.m_slots, hand_back, landed);
+    }
 
   const bool leader = p.regime == 0 || warp % (kWarps / p.groups) == 0;  // holds window accumulators
   if (BASE && leader) flush_base(p, S, bacc, lane);

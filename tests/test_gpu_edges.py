@@ -290,3 +290,22 @@ def test_rank_bracket_at_word_end(sf, T, R, S, relative, late):
     assert int(st.item()) == 0
     assert np.array_equal(host(g.L), o.L) and np.array_equal(host(g.dL), o.dL) and np.array_equal(host(g.G), o.G)
     assert np.array_equal(host(sp), O.raw_spread(d_np, 4, 3))
+
+
+# medians that stay in shared memory, in one slot and in two: CTA ranges of 25 steps that
+# start and end at every place of windows of 24 (on a window's last step, one step into the
+# next), whole-row steps and ragged ones, without and with the quality sums
+@pytest.mark.parametrize("R,S", [(512, 10), (1001, 5), (300, 10), (700, 12)])
+def test_resident_medians_at_range_edges(sf, R, S):
+    T, W = 25 * torch.cuda.get_device_properties(0).multi_processor_count, 24
+    d_np = durations(T, R, S, "ms", R)
+    d, m_np = dev(d_np), O.window_median(d_np, W)
+    m, st = dev(m_np), sf.new_status("cuda")
+    X, Y = O.windows(d_np, W).X, O.direct_gain(d_np, W, m_np)
+    wall = dev(d_np.sum(axis=2) + 1000)
+    for _ in range(8):
+        ev = sf.sf_direct_gain(d, W, m, status=st)
+        assert np.array_equal(host(ev.X), X) and np.array_equal(host(ev.Y), Y)
+        ev = sf.sf_direct_gain(d, W, m, wall=wall, status=st)
+        assert np.array_equal(host(ev.X), X) and np.array_equal(host(ev.Y), Y)
+    assert int(st.item()) == 0
