@@ -309,3 +309,117 @@ def test_resident_medians_at_range_edges(sf, R, S):
         ev = sf.sf_direct_gain(d, W, m, wall=wall, status=st)
         assert np.array_equal(host(ev.X), X) and np.array_equal(host(ev.Y), Y)
     assert int(st.item()) == 0
+
+
+def evidence(d, W, wall=None, other=-1):
+    """What sf_direct_gain reports beside the oracle's sums: the leader byte with its
+    confidence at eta_Q = 1/20, and the quality sums (residual, overlap, wall)."""
+    P = d.cumsum(axis=2)
+    F = P.max(axis=1)
+    a = np.diff(F, axis=1, prepend=0)
+    best = a.argmax(axis=1)
+    rest = a.copy()
+    rest[np.arange(len(a)), best] = 0
+    sure = (F[:, -1] > 0) & ((a.max(axis=1) - rest.max(axis=1)) * 20 >= F[:, -1])
+    o = d[:, :, other] if other >= 0 else np.zeros(d.shape[:2], np.int64)
+    if wall is None:
+        sums = (o, np.zeros_like(o), P[:, :, -1])
+    else:
+        e = wall - (P[:, :, -1] - o)
+        sums = (np.maximum(e, 0), np.maximum(-e, 0), wall)
+    q = [[sum(map(int, x[t:t + W].sum(axis=1))) for x in sums] for t in range(0, len(d), W)]
+    return (best | np.where(sure, 128, 0)).astype(np.uint8), q
+
+
+def check_evidence(sf, d_np, W, options, place=dev):
+    """Every form of the pass in `options` (wall, other_stage); place: medians to the device."""
+    d, st = dev(d_np), sf.new_status("cuda")
+    m_np, ow = O.window_median(d_np, W), O.windows(d_np, W)
+    m, Y = place(m_np), O.direct_gain(d_np, W, m_np)
+    for wall, other in options:
+        ev = sf.sf_direct_gain(d, W, m, wall=None if wall is None else dev(wall), other_stage=other, lead_credit=True,
+                               status=st)
+        assert int(st.item()) == 0
+        assert np.array_equal(host(ev.X), ow.X) and np.array_equal(host(ev.Y), Y) and np.array_equal(host(ev.D), ow.D)
+        assert np.array_equal(host(ev.E), ow.E) and np.array_equal(host(ev.C), ow.C)
+        lead, q = evidence(d_np, W, wall, other)
+        assert np.array_equal(host(ev.step_lead), lead)
+        if wall is not None or other >= 0:
+            got = host(ev.quality.view(torch.int64)).astype(object) & ((1 << 64) - 1)
+            assert [[int(w[2 * i]) | int(w[2 * i + 1]) << 64 for i in range(3)] for w in got] == q
+
+
+# steps enough for a lane per (step, stage): every scan depth, one to 16 steps a tile, a
+# partial last tile and window, steps past 32 bits, sums past 64
+LANES = [(20000, 3, 1, 999), (9001, 60, 2, 500), (6000, 7, 6, 250), (4000, 33, 13, 300), (3000, 100, 16, 3000),
+         (2600, 64, 11, 2600), (1300, 12, 24, 100), (700, 9, 32, 64), (650, 130, 17, 50)]
+
+
+@pytest.mark.parametrize("T,R,S,W", LANES)
+@pytest.mark.parametrize("kind", ["ms", "long", "huge"])
+def test_step_lanes(sf, T, R, S, W, kind):
+    d_np = durations(T, R, S, "long" if kind == "long" else "ms", T + R)
+    if kind == "huge":
+        d_np = np.minimum(d_np * (1 << 17), (1 << 46) // S)
+    rng = np.random.default_rng(T)
+    wall = d_np.sum(axis=2) + rng.integers(-100000, 100000, size=(T, R))
+    check_evidence(sf, d_np, W, [(None, -1), (wall, -1), (wall, S - 1), (None, S // 2)])
+    d, st = dev(d_np), sf.new_status("cuda")
+    b, ob = sf.sf_window_baselines(d, W, status=st), O.baselines(d_np, W)
+    s2 = host(b.SUM.view(torch.int64)).astype(object) & ((1 << 64) - 1)
+    assert (s2[..., 0] + (s2[..., 1] << 64) == ob.SUM).all()
+    assert np.array_equal(host(b.M), ob.M) and np.array_equal(host(b.SLOW), ob.SLOW)
+    assert np.array_equal(host(b.RANK0), ob.RANK0)
+    f, o = sf.sf_frontier(d, status=st), O.frontier(d_np)
+    assert np.array_equal(host(f.a), o.a) and np.array_equal(host(f.lead), o.lead)
+    assert np.array_equal(host(f.makespan), o.makespan) and int(st.item()) == 0
+
+
+# medians that are only 8-byte aligned: steps of many and of few ranks, few steps and many
+@pytest.mark.parametrize("T,R,S,W", [(5000, 31, 7, 500), (5000, 130, 4, 500), (300, 40, 6, 50), (12, 1500, 10, 4)])
+@pytest.mark.parametrize("kind", ["ms", "long"])
+def test_unaligned_medians(sf, T, R, S, W, kind):
+    def place(m_np):
+        buf = torch.empty(m_np.size + 1, dtype=torch.int64, device="cuda")
+        buf[1:] = torch.from_numpy(m_np).cuda().view(-1)
+        m = buf[1:].view(m_np.shape)
+        assert m.data_ptr() % 16 == 8
+        return m
+    d_np = durations(T, R, S, kind, T + R)
+    check_evidence(sf, d_np, W, [(None, -1), (d_np.sum(axis=2) + 1000, 0)], place)
+
+
+# durations and totals out of range are flagged by every form: lanes, warps, tiles and CTAs
+@pytest.mark.parametrize("T,R,S", [(6000, 7, 6), (700, 9, 32), (2000, 60, 16), (40, 16, 8), (30, 100, 8), (30, 100, 9),
+                                   (9, 300, 5), (4, 3000, 4), (3, 8192, 8), (2, 5000, 13), (100, 128, 8), (300, 200, 3),
+                                   (10001, 9, 2)])
+def test_status_bits_of_every_form(sf, T, R, S):
+    group = dev(np.zeros(R, np.int32))
+    calls = dict(frontier=lambda d, st: sf.sf_frontier(d, status=st),
+                 ties=lambda d, st: sf.sf_frontier_ties(d, a=torch.zeros((T, S), dtype=torch.int64, device="cuda"), status=st),
+                 windows=lambda d, st: sf.sf_window_aggregate(d, 50, status=st),
+                 baselines=lambda d, st: sf.sf_window_baselines(d, 50, status=st),
+                 gain=lambda d, st: sf.sf_direct_gain(d, 50, torch.ones((-(-T // 50), R, S), dtype=torch.int64, device="cuda"), status=st),
+                 lag=lambda d, st: sf.sf_rank_lag(d, status=st), spread=lambda d, st: sf.sf_raw_spread(d, 50, status=st),
+                 groups=lambda d, st: sf.sf_group_aggregate(d, group, 1, 50, status=st))
+    at = (T * 2 // 3, R * 3 // 4, S // 2)
+    for values, bit in (({at: -5}, sf.SF_ST_NEGATIVE), ({at: 1 << 47}, sf.SF_ST_RANGE),
+                        ({at[:2] + (0,): 1 << 46, at[:2] + (S - 1,): 1 << 46}, sf.SF_ST_RANGE),
+                        ({at: (1 << 47) - 1 - S}, 0)):
+        d_np = np.ones((T, R, S), np.int64)
+        for i, v in values.items():
+            d_np[i] = v
+        d = dev(d_np)
+        for name, call in calls.items():
+            if name == "spread" and len(values) == 2:
+                continue  # durations only
+            st = sf.new_status("cuda")
+            call(d, st)
+            assert int(st.item()) & 3 & (bit or 3) == bit, (name, values)
+    wall = np.ones((T, R), np.int64)
+    m = torch.ones((-(-T // 50), R, S), dtype=torch.int64, device="cuda")
+    for v, bit in ((-1, sf.SF_ST_NEGATIVE), (1 << 47, sf.SF_ST_RANGE)):
+        wall[at[:2]] = v
+        st = sf.new_status("cuda")
+        sf.sf_direct_gain(dev(np.ones((T, R, S), np.int64)), 50, m, wall=dev(wall), status=st)
+        assert int(st.item()) & bit
