@@ -305,23 +305,34 @@ __global__ void __launch_bounds__(kGlThreads, 5) group_lanes_kernel(const __grid
   int64_t w = -1, w_end = 0;  // window of the lane's step: steps below w_end
   bool wide = false;          // walk the next tile in 64 bits at once
   for (int g = 0; g < G; ++g) acc[g * 32 + lane] = 0;
+  // The warp's window sums to global memory, those of one window over its steps first
+  // (two atomics for every lane and group: 100000 x 128 x 3, 16 groups, 157 -> 115 us).
   auto flush = [&]() {
-    if (w < 0) return;
+    const bool one = one_window(w);
     for (int g = 0; g < G; ++g) {
-      const int64_t x = acc[g * 32 + lane];
-      if (x == 0) continue;
+      int64_t x = acc[g * 32 + lane], all;
       acc[g * 32 + lane] = 0;
-      atomicAdd(reinterpret_cast<unsigned long long*>(&p.Xg[(w * G + g) * S + s]), static_cast<unsigned long long>(x));
-      // the increments of a step add up to its makespan
-      atomicAdd(reinterpret_cast<unsigned long long*>(&p.Dg[w * G + g]), static_cast<unsigned long long>(x));
+      if (one) x = sum_steps(x, S, lane);
+      all = x;  // the increments of a step add up to its makespan
+      if (one)
+        for (int o = 1; o < S; o <<= 1) {
+          const int64_t up = __shfl_down_sync(kFull, all, o);
+          if (lane + o < S) all += up;
+        }
+      if (w < 0 || (one && lane >= S)) continue;
+      if (x != 0)
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.Xg[(w * G + g) * S + s]), static_cast<unsigned long long>(x));
+      if (all != 0 && (!one || lane == 0))
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.Dg[w * G + g]), static_cast<unsigned long long>(all));
     }
   };
   for (int64_t tile = tiles * id / nw; tile < tile_end; ++tile) {
     const int64_t t0 = tile * steps;
     const bool live = j < steps && t0 + j < p.T;
     const int64_t t = live ? t0 + j : t0;
-    if (live && (w < 0 || t >= w_end)) {
-      flush();
+    const bool next = live && (w < 0 || t >= w_end);
+    if (__any_sync(kFull, next && w >= 0)) flush();
+    if (next) {
       w = (p.t0 + t) / p.W - p.w_first;
       w_end = (w + p.w_first + 1) * p.W - p.t0;
     }

@@ -1,5 +1,6 @@
-// sf_lane_select.cuh - selection by single lanes, each on a column of up to 128
-// keys that it holds in registers, its loads spread over the warp's 32 columns.
+// sf_lane_select.cuh - kernels that give a lane a (step, stage) or a column: loads,
+// sums over a warp's steps, and selection by single lanes, each on a column of up to
+// 128 keys that it holds in registers, its loads spread over the warp's 32 columns.
 #pragma once
 
 #include "sf_device.cuh"
@@ -18,6 +19,32 @@ __device__ __forceinline__ uint2 load_words(const int64_t* p) {
   uint2 v;
   asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
   return v;
+}
+
+// Lanes j S + s hold stage s of a warp's j-th step (0 on lanes past the last whole
+// step): the sum over the steps, on lanes s < S.  The whole warp calls it.
+__device__ __forceinline__ int64_t sum_steps(int64_t v, int S, int lane) {
+  for (int o = S; o < 32; o <<= 1) {
+    const int64_t up = __shfl_down_sync(kFull, v, o);
+    if (lane + o < 32) v += up;
+  }
+  return v;
+}
+__device__ __forceinline__ unsigned __int128 sum_steps(unsigned __int128 v, int S, int lane) {
+  uint64_t lo = static_cast<uint64_t>(v), hi = static_cast<uint64_t>(v >> 64);
+  for (int o = S; o < 32; o <<= 1) {
+    const uint64_t l = __shfl_down_sync(kFull, lo, o), h = __shfl_down_sync(kFull, hi, o);
+    if (lane + o < 32) {
+      lo += l;
+      hi += h + (lo < l ? 1u : 0u);
+    }
+  }
+  return (static_cast<unsigned __int128>(hi) << 64) | lo;
+}
+// Whether the warp's lanes (w < 0: none yet) are all in the first one's window.
+__device__ __forceinline__ bool one_window(int64_t w) {
+  const int64_t first = __shfl_sync(kFull, w, 0);
+  return __all_sync(kFull, w == first || w < 0);
 }
 
 // The kth (from 0) smallest of this lane's n keys (the others hold 0xffffffff),

@@ -195,6 +195,15 @@ def test_group_lanes(sf, T, R, S, G, kind):
     assert np.array_equal(host(g.X), np.transpose(o.X, (1, 0, 2))) and np.array_equal(host(g.D), o.D.T)
 
 
+# the same where the lanes have many tiles each: windows that end within a tile, the
+# largest rank and group counts, stages in the lanes' every layout
+@pytest.mark.parametrize("T,R,S,G", [(100001, 20, 1, 3), (60000, 192, 3, 2), (30000, 40, 4, 1), (40000, 65, 8, 32),
+                                     (6000, 31, 10, 7), (12000, 50, 13, 4), (9000, 20, 24, 6)])
+@pytest.mark.parametrize("kind", ["blocks", "mixed", "long"])
+def test_group_lanes_many_steps(sf, T, R, S, G, kind):
+    test_group_lanes(sf, T, R, S, G, kind)
+
+
 # small steps: windows of a tile's 16 steps and one less and more, a short last
 # window, a tile of ranks and one more, the largest small step and the next
 @pytest.mark.parametrize("T,R,S,N", [(100, 16, 8, 16), (95, 31, 7, 15), (100, 47, 8, 17), (1000, 48, 8, 100),
