@@ -20,6 +20,7 @@
 // parking it in shared memory when the group changes, so no lane waits for
 // another before the step's end.
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <type_traits>
 
@@ -223,10 +224,29 @@ __global__ void __launch_bounds__(kGrThreads) group_window_kernel(const GroupPar
 constexpr int kGlThreads = 128;
 constexpr int kGlWarps = kGlThreads / 32;
 constexpr int kGlBatch = 8;
-constexpr int kGlMaxGroups = 32;
-// (us, CTA per step / lanes: 100000 x 16 x 8 461 / 72, 100000 x 31 x 7 563 / 82,
-// 131072 x 64 x 16 753 / 309, 100000 x 128 x 8 352 / 254, 50000 x 300 x 6 237 / 271)
+constexpr int64_t kGlMaxGroups = 32;
 constexpr int64_t kGlMaxRanks = 192;
+constexpr int64_t group_lanes_smem(int64_t G) { return kGlWarps * 2 * G * 32 * 8; }  // at most 64 KB
+
+// Whether the lanes take a call, by estimates of both forms' time in us.  A warp's walk
+// is a chain of loads and scans per rank, and of one exchange per group at a step's end:
+// with few tiles of steps per warp it is slower than a CTA per step (1500 x 128 x 8 in
+// node groups 14 us, 41 by lanes).  Fitted to 1866 measured calls of 700 to 100000
+// steps, 4 to 192 ranks, 1 to 24 groups (lanes within 10 %, CTAs within 20 %).  Steps
+// past 32 bits take the lanes up to twice as long, so they are taken when they are
+// half as fast again: then no call of ordinary steps was slower by more than 5 % and 45 of
+// 1866 of steps past 32 bits were (at most 1.55 times; all together 2.1 times as fast).
+bool use_group_lanes(int64_t T, int64_t R, int64_t S, int64_t G) {
+  if (R > kGlMaxRanks || G > kGlMaxGroups) return false;
+  const double sms = sm_count();
+  const double per_cta = static_cast<double>((T + 32 / S - 1) / (32 / S)) / (sms * kGlWarps);  // tiles, one CTA per SM
+  if (per_cta < 1.0) return false;
+  const double ctas = static_cast<double>(std::min<int64_t>(5, 227 * 1024 / (group_lanes_smem(G) + 1024)));
+  const double rounds = std::ceil(per_cta / ctas);
+  const double lanes = 9.0 + rounds * (0.45 + 0.092 * R + 0.53 * G) + per_cta * (0.020 * R + 0.017 * G);
+  const double cta = 9.1 + T / (8.0 * sms) * (0.99 + 0.37 * S + 0.018 * G * S + (G > 1 ? 0.126 * S : 0.0));
+  return 1.5 * lanes < cta;
+}
 
 // Walks the ranks of a warp's steps: park[g][lane] becomes the lane's stage of
 // F_g.  32-bit prefixes unless WIDE; returns whether they hold.
@@ -361,7 +381,7 @@ __global__ void __launch_bounds__(kGlThreads, 5) group_lanes_kernel(const __grid
 template <int LOGS>
 cudaError_t launch_group_lanes(const GroupParams& p, cudaStream_t stream) {
   auto kern = group_lanes_kernel<LOGS>;
-  const size_t smem = size_t(kGlWarps) * 2 * p.G * 32 * 8;  // at most 64 KB
+  const size_t smem = static_cast<size_t>(group_lanes_smem(p.G));
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   int per_sm = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGlThreads, smem);
@@ -447,7 +467,7 @@ cudaError_t launch_group_windows(const int64_t* d, int64_t T, int64_t R, int64_t
   p.Xg = Xg;
   p.Dg = Dg;
   p.status = status;
-  if (R <= kGlMaxRanks && G <= kGlMaxGroups && (T + 32 / S - 1) / (32 / S) >= int64_t(sm_count()) * 4) {
+  if (use_group_lanes(T, R, S, G)) {
     if (S <= 1) return launch_group_lanes<0>(p, stream);
     if (S <= 2) return launch_group_lanes<1>(p, stream);
     if (S <= 4) return launch_group_lanes<2>(p, stream);
