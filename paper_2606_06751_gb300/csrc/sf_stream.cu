@@ -530,17 +530,49 @@ namespace {
 
 // One lane per (step, stage) instead of tiles: small steps, whose S warp
 // reductions each outweigh their few rank rows, and the evidence pass over more
-// stages than the tiles take.  Measured on 0.1 to 1.1 GB, tiles against lanes, us:
-// evidence 16 x 8 88 / 39, 64 x 16 422 / 269, 64 x 8 115 / 111, 128 x 16 111 / 95,
-// 128 x 8 164 / 202, 256 x 8 239 / 246; baselines 64 x 8 114 / 88, 128 x 8 144 / 164;
-// frontier 12 x 3 133 / 38, 31 x 7 61 / 47, 128 x 6 102 / 131; evidence 1000 x 24
-// 570 (a CTA per step) / 183.  The warps (20 per SM) need steps enough to go round.
+// stages than the tiles take.  A warp walks its steps' ranks one after another, so
+// the warps (20 per SM) need steps enough to go round, and a step past 32 bits, walked
+// in 64, takes about twice as long where the other forms lose a fifth.  The rank limits
+// are where the lanes no longer gain on ordinary steps what half as many long ones
+// would lose.  Us, the best other form / lanes, for ordinary steps and, in brackets,
+// the same times 64:
+//   frontier              48000 x 16 x 6    26.7 / 12.4 (26.7 / 20.5)
+//                         48000 x 48 x 6    32.8 / 32.4 (33.0 / 51)
+//   baselines             48000 x 64 x 8      62 / 46   (62 / 79)
+//                         24000 x 64 x 16     53 / 46   (53 / 84)
+//                         24000 x 48 x 12   39.5 / 36.8 (39.2 / 66)
+//   evidence              24000 x 64 x 16     93 / 55   (97 / 109)
+//                         24000 x 64 x 8    34.9 / 30.6 (51 / 59)
+//                         24000 x 64 x 10     42 / 43   (51 / 85)
+//                         608 x 96 x 20     26.7 / 14.3 (27.0 / 29.9), a CTA per step / lanes
+//                         608 x 1000 x 20     92 / 110  (92 / 316)
+//                         1500 x 1000 x 20   251 / 130  (250 / 374)
+//   with quality sums     24000 x 16 x 10     53 / 33.8 (63 / 56)
+//                         24000 x 48 x 16    127 / 88   (127 / 164)
+//                         24000 x 32 x 12     49 / 65   (49 / 116)
+//                         2500 x 192 x 24    131 / 90   (131 / 220)
+//                         2500 x 192 x 20    105 / 88   (105 / 214)
+//                         9000 x 192 x 20    367 / 251  (368 / 499)
+//   medians only 8-byte   10000 x 64 x 6    22.5 / 14.5 (22.6 / 30.8)
+//   aligned               5000 x 64 x 4     12.4 / 10.3 (12.3 / 16.5)
+//                         20000 x 64 x 6      40 / 54   (40 / 111), with quality sums
 bool use_step_lanes(int kind, int64_t T, int64_t R, int64_t S, bool fast, int sms) {
-  if (S <= 16 && !fast) return T >= int64_t(sms) * 32;  // medians only 8-byte aligned
-  if ((T + 32 / S - 1) / (32 / S) < int64_t(sms) * 4) return false;
-  if (kind == kFrontier) return S <= 16 && lanes_groups(R, S) == 0 && R * S * 8 <= 3072;
-  if (S > 16) return is_gain(kind);
-  return R <= 64 || (S == 16 && R <= 128);
+  const int64_t tiles = (T + 32 / S - 1) / (32 / S);
+  if (tiles < int64_t(sms) * 4) return false;
+  if (S > 16) {  // against a CTA per step
+    if (kind == kGain) return R <= 192 || T >= int64_t(sms) * (S > 24 ? 4 : 10);
+    if (kind != kGainQuality) return false;
+    return S >= 24 ? T * S >= int64_t(sms) * 384 : R <= 192 && T >= int64_t(sms) * (R <= 96 ? 10 : 30);
+  }
+  if (!fast)  // against a CTA per step
+    return T >= int64_t(sms) * 32 && tiles >= int64_t(sms) * 8 && (kind != kGainQuality || S == 16 || R <= 16);
+  const bool full = S <= 4 || S == 8 || S == 16;  // few or none of the lanes idle
+  switch (kind) {
+    case kFrontier: return lanes_groups(R, S) == 0 && R <= (S <= 8 ? 48 : 32) && R * S * 8 <= 3072;
+    case kBase: return R <= (S <= 8 ? 64 : S <= 11 || S == 16 ? 48 : 32);
+    case kGain: return R <= (S == 16 ? 128 : full ? 64 : S <= 11 ? 48 : 32);
+    default: return R <= 16 || (R <= 48 && full && tiles >= int64_t(sms) * 16);
+  }
 }
 
 // Whether the evidence pass keeps whole windows of medians (`rows` 128-byte

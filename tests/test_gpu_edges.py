@@ -361,7 +361,10 @@ def check_evidence(sf, d_np, W, options, place=dev):
 # steps enough for a lane per (step, stage): every scan depth, one to 16 steps a tile, a
 # partial last tile and window, steps past 32 bits, sums past 64
 LANES = [(20000, 3, 1, 999), (9001, 60, 2, 500), (6000, 7, 6, 250), (4000, 33, 13, 300), (3000, 100, 16, 3000),
-         (2600, 64, 11, 2600), (1300, 12, 24, 100), (700, 9, 32, 64), (650, 130, 17, 50)]
+         (2600, 64, 11, 2600), (1300, 12, 24, 100), (700, 9, 32, 64), (650, 130, 17, 50),
+         # the most ranks that a pass takes by lanes, and the fewest steps
+         (6000, 48, 6, 333), (9800, 48, 8, 700), (2600, 48, 11, 2600), (4000, 32, 13, 300), (4000, 16, 14, 250),
+         (4900, 48, 16, 500), (1530, 96, 17, 50), (4600, 97, 17, 500), (2500, 130, 24, 100)]
 
 
 @pytest.mark.parametrize("T,R,S,W", LANES)
