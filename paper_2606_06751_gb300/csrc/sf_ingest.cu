@@ -65,10 +65,26 @@ constexpr int kTileBytes = 48 * 1024;
 // values of a rank's run in the tile, padded to an odd number against bank conflicts
 __host__ __device__ constexpr int tile_pitch(int S) { return kTileSteps * S | 1; }
 
-// Steps a CTA has little to do for (us before and with tiles: 100000 x 16 x 8 102 /
-// 45, 100000 x 31 x 7 161 / 90); larger ones move as fast or faster directly
-// (100000 x 128 x 8 262 / 292, 13421 x 1000 x 5 230 / 235, 8192 x 8 358 / 371).
-bool use_tiles(int64_t R, int64_t S, int64_t N) { return N >= kTileSteps && R * S * 8 <= 3072; }
+struct IngestTiles {
+  int ranks = 0;      // of a tile; 0: no tiles
+  int64_t count = 0;
+};
+
+// Steps a CTA has little to do for, and tiles for every SM (us, directly / tiles:
+// 100000 x 16 x 8 102.6 / 44.8, 100000 x 31 x 7 160 / 90, 20000 x 64 x 5 53.5 / 27.3;
+// 1500 x 32 x 6, of 94 tiles, 4.1 / 6.2).  Odd stage counts, moved 8 bytes at a time
+// directly, gain up to 3 KB a step; even ones, moved 16 bytes, up to 2.5 KB and 64 ranks
+// (100000 x 64 x 4 117 / 101, 96 x 4 130 / 150, 32 x 12 125 / 122, 128 x 2 117 / 143).
+IngestTiles plan_tiles(int64_t T, int64_t R, int64_t S, int64_t N) {
+  IngestTiles p;
+  const bool small = S % 2 == 0 ? R <= 64 && R * S <= 320 : R <= (S == 1 ? 96 : 128) && R * S <= 384;
+  if (N < kTileSteps || !small) return p;
+  // even shares of the ranks (100000 x 64 x 6, whose tiles hold 63 ranks: 63 and 1 206 us, 32 and 32 125)
+  const int64_t most = kTileBytes / (8 * tile_pitch(static_cast<int>(S))), blocks = (R + most - 1) / most;
+  p.count = (T + N - 1) / N * ((N + kTileSteps - 1) / kTileSteps) * blocks;
+  if (p.count >= sm_count()) p.ranks = static_cast<int>((R + blocks - 1) / blocks);
+  return p;
+}
 
 __global__ void __launch_bounds__(kIngThreads) gathered_tiles_kernel(const int64_t* __restrict__ src, int64_t T,
                                                                      int64_t R, int S, int64_t N, int ranks,
@@ -117,12 +133,10 @@ __global__ void __launch_bounds__(kIngThreads) gathered_tiles_kernel(const int64
 cudaError_t launch_gathered_to_steps(const int64_t* src, int64_t T, int64_t R, int64_t S, int64_t N, int64_t* dst,
                                      cudaStream_t stream) {
   N = std::min(N, T);  // one window holds them all
-  if (use_tiles(R, S, N)) {
-    const int ranks = static_cast<int>(std::min<int64_t>(R, kTileBytes / (8 * tile_pitch(static_cast<int>(S)))));
-    const int64_t tiles = (T + N - 1) / N * ((N + kTileSteps - 1) / kTileSteps) * ((R + ranks - 1) / ranks);
-    const int grid = static_cast<int>(std::min<int64_t>(tiles, int64_t(sm_count()) * 4));
+  if (const IngestTiles tiles = plan_tiles(T, R, S, N); tiles.ranks > 0) {
+    const int grid = static_cast<int>(std::min<int64_t>(tiles.count, int64_t(sm_count()) * 4));
     count_launch();
-    gathered_tiles_kernel<<<grid, kIngThreads, 0, stream>>>(src, T, R, static_cast<int>(S), N, ranks, dst);
+    gathered_tiles_kernel<<<grid, kIngThreads, 0, stream>>>(src, T, R, static_cast<int>(S), N, tiles.ranks, dst);
     return cudaGetLastError();
   }
   const int unit = S % 2 == 0 ? 2 : 1;
