@@ -828,7 +828,8 @@ cudaError_t launch_rank_select(const int64_t* d, int64_t T, int64_t R, int64_t S
                                int64_t W, int64_t* L, int64_t* dL, int64_t* G, int64_t* Lw, int64_t* Gw,
                                int64_t* spread, void* workspace, size_t ws_bytes, uint32_t* status,
                                cudaStream_t stream) {
-  if (rank_on_chip(R, S)) return launch_rank_chip(d, T, R, S, of_prefix, t0, W, L, dL, G, Lw, Gw, spread, status, stream);
+  if (rank_on_chip(T, R, S))
+    return launch_rank_chip(d, T, R, S, of_prefix, t0, W, L, dL, G, Lw, Gw, spread, status, stream);
   const size_t half = ws_bytes / 2 & ~size_t(255);  // one chunk buffer, 256-byte aligned
   const int64_t Tc = chunk_steps_for(T, R, S, half);
   if (Tc < 1) return cudaErrorInvalidValue;

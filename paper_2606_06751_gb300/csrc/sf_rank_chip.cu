@@ -4,8 +4,8 @@
 // value.  d is read once and nothing is written but the results; sf_rank.cu
 // takes the larger steps through a scratch in L2.
 //
-// Which kernel takes a step, and what each measured as lag over 0.1 to 4.1 GB
-// against the passes through L2 (whose per-column CTAs have little to do on few
+// Which kernel takes a call (rank_form), and what each measured as lag over 0.1 to
+// 4.1 GB against the passes through L2 (whose per-column CTAs have little to do on few
 // ranks):
 //  rank_lanes_kernel (sf_rank_lanes.cu) - up to 128 ranks: one lane per column,
 //    its keys in registers (100000 x 16 x 8 3133 -> 44 us, 131072 x 64 x 16
@@ -20,11 +20,11 @@
 //    then holds a column in registers and searches it by a radix selection, 8
 //    bits a pass, or by counting.  Bound by the chain of loads, barrier and
 //    selection, which resident CTAs overlap (50000 x 1024 x 10: 3567 -> 1118 us,
-//    60000 x 256 x 8 442 us).
+//    60000 x 256 x 8 442 us).  It also takes few steps of up to 128 ranks.
 //  rank_step_kernel - the same for more ranks, one to eight warps per column
 //    reading the keys from shared memory in each pass (10000 x 4000 x 3:
-//    1247 -> 492 us; 5000 x 2800 x 8, at the limit of two CTAs per SM, 454 ->
-//    448 us: beyond it the passes through L2 are as good).
+//    1247 -> 492 us; with eight stages it would be as slow as the passes
+//    through L2: 600 x 2500 x 8 56 / 60 us, of long steps 62 / 83).
 //
 // Keys are the values' low words.  A step whose values all fit 32 bits (rank
 // totals below 4.29 s) orders by them as they are; otherwise the step is read
@@ -496,12 +496,37 @@ cudaError_t launch_column(ChipParams p, cudaStream_t stream) {
                       : launch_chip(rank_column_kernel<NPL, false>, p, threads, smem, 1, stream);
 }
 
+// The form of a call's steps.  The lines, with lag in us, also of steps 64 times as long
+// (in brackets), through L2 / by the form the line is drawn against / by the form chosen:
+//  - Few steps of up to 128 ranks leave the lanes a tile or two per warp, and one past 32
+//    bits, which its warp takes again column by column, waits for nothing else: a CTA per
+//    step up to 10 steps per SM (300 x 64 x 4 14.4 / 10.3 / 6.2 (16.5 / 75.8 / 8.3),
+//    1500 x 64 x 8 57.9 / 10.3 / 12.3 (58.7 / 76.9 / 16.4)).
+//  - The column form has a warp per stage, too few to load few steps of many ranks and few
+//    stages: those take the step form (40 x 1024 x 1 13.3 / 14.4 / 7.6, 300 x 2048 x 1
+//    20.5 / 23.6 / 8.3, against 1500 x 1024 x 1 38.2 / 14.4 / 22.6).
+//  - With more stages few large steps leave SMs idle that the passes through L2 use:
+//    20 x 2048 x 10 16.4 / 20.5, 80 x 2048 x 10 22.6 / 20.6; 40 x 3000 x 6 16.4 / 20.5,
+//    300 x 3000 x 6 30.8 / 26.7.
+enum RankForm { kRankPasses, kRankLanes, kRankWarp, kRankColumn, kRankStep };
+
+RankForm rank_form(int64_t T, int64_t R, int64_t S) {
+  const int64_t sms = sm_count();
+  if (R <= kRankLaneMax) {
+    if (T < sms * 10) return kRankColumn;
+    return R >= kRankWarpMin && S <= kRankWarpMaxS ? kRankWarp : kRankLanes;
+  }
+  const bool step = step_smem(R, S) <= kStepSmemMax;
+  if (R <= kColMaxRanks && column_smem(R, S) <= kStepSmemMax) {
+    if (step && (S <= 2 ? R > 256 && T < sms * 4 : S <= 4 && R > 1024 && T < sms * 2)) return kRankStep;
+    return S > 8 && R > 1024 && T < sms / 2 ? kRankPasses : kRankColumn;
+  }
+  return step && S != 8 && (S <= 4 || T >= sms) ? kRankStep : kRankPasses;
+}
+
 }  // namespace
 
-bool rank_on_chip(int64_t R, int64_t S) {
-  return R <= kRankLaneMax || (R <= kColMaxRanks && column_smem(R, S) <= kStepSmemMax) ||
-         step_smem(R, S) <= kStepSmemMax;
-}
+bool rank_on_chip(int64_t T, int64_t R, int64_t S) { return rank_form(T, R, S) != kRankPasses; }
 
 cudaError_t launch_rank_chip(const int64_t* d, int64_t T, int64_t R, int64_t S, int of_prefix, int64_t t0, int64_t W,
                              int64_t* L, int64_t* dL, int64_t* G, int64_t* Lw, int64_t* Gw, int64_t* spread,
@@ -522,9 +547,11 @@ cudaError_t launch_rank_chip(const int64_t* d, int64_t T, int64_t R, int64_t S, 
   p.Gw = Gw;
   p.spread = spread;
   p.status = status;
-  if (R >= kRankWarpMin && R <= kRankLaneMax && S <= kRankWarpMaxS) return launch_rank_warp(p, stream);
-  if (R <= kRankLaneMax) return launch_rank_lanes(p, stream);
-  if (R <= kColMaxRanks && column_smem(R, S) <= kStepSmemMax) {
+  const RankForm form = rank_form(T, R, S);
+  if (form == kRankPasses) return cudaErrorInvalidValue;
+  if (form == kRankWarp) return launch_rank_warp(p, stream);
+  if (form == kRankLanes) return launch_rank_lanes(p, stream);
+  if (form == kRankColumn) {
     if (R <= 256) return launch_column<8>(p, stream);
     if (R <= 512) return launch_column<16>(p, stream);
     if (R <= 1024) return launch_column<32>(p, stream);

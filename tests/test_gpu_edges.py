@@ -136,6 +136,19 @@ def test_rank_on_chip(sf, T, R, S, kind):
     assert np.array_equal(host(Lw), oL) and np.array_equal(host(Gw), oG)
 
 
+# the forms that take many steps (lanes, warps), and the lines between the others: stages
+# and steps on both sides of each
+@pytest.mark.parametrize("T,R,S", [(1600, 1, 4), (1519, 40, 3), (1520, 40, 3), (1600, 16, 8), (1601, 17, 16), (1700, 32, 17),
+                                   (1600, 33, 17), (1600, 64, 9), (1600, 65, 16), (1600, 65, 8), (1600, 104, 10),
+                                   (1530, 105, 32), (1600, 128, 8), (1600, 128, 9), (1600, 100, 5),
+                                   (607, 300, 2), (608, 300, 2), (303, 1025, 3), (304, 1025, 3), (310, 2048, 4),
+                                   (700, 1500, 1), (75, 1100, 9), (76, 2048, 9), (7, 2048, 7), (20, 1100, 6),
+                                   (151, 2893, 6), (152, 2893, 6), (153, 2050, 11)])
+@pytest.mark.parametrize("kind", ["ms", "long", "far", "tail", "halves"])
+def test_rank_forms(sf, T, R, S, kind):
+    test_rank_on_chip(sf, T, R, S, kind)
+
+
 # steps that are not whole 128-byte rows: every stage count, small steps (whole
 # steps per tile) and steps of one or more tiles with one, two and four warp
 # groups, a tensor and medians that end inside a row, tensors below one row;
@@ -290,7 +303,8 @@ def test_gathered_pieces(sf, T, R, S, N):
 
 # columns in shared memory whose median lies in the last bins below 2^32, by their
 # values and relative to rank 0: one to eight warps per column
-@pytest.mark.parametrize("T,R,S", [(6, 4000, 3), (5, 2500, 6), (4, 9000, 2), (5, 2050, 11), (3, 11001, 1), (200, 3000, 4)])
+@pytest.mark.parametrize("T,R,S", [(6, 4000, 3), (160, 2500, 6), (4, 9000, 2), (160, 2050, 11), (3, 11001, 1),
+                                   (200, 3000, 4)])
 @pytest.mark.parametrize("relative", [False, True])
 @pytest.mark.parametrize("late", [1 << 23, 64])
 def test_rank_bracket_at_word_end(sf, T, R, S, relative, late):
