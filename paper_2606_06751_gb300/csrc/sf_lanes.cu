@@ -113,12 +113,10 @@ __global__ void __launch_bounds__((kLaneWarps + kProducers) * 32, 1)
   const int64_t NB = gridDim.x, b = blockIdx.x;
   const int64_t t_begin = p.T * b / NB, t_end = p.T * (b + 1) / NB;
 
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < kMaxStages; ++i) {
-      mbar_init(&full[i], 1);
-      mbar_init(&empty[i], 1);
-    }
-    *abort = 0;
+  if (threadIdx.x < kMaxStages) {
+    mbar_init(&full[threadIdx.x], 1);
+    mbar_init(&empty[threadIdx.x], 1);
+    if (threadIdx.x == 0) *abort = 0;
     fence_barrier_init();
   }
   __syncthreads();

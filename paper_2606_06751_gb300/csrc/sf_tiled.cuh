@@ -224,16 +224,14 @@ __global__ void __launch_bounds__((consumer_warps(KIND, S) + kProducers) * 32, 1
   const int64_t G = gridDim.x, b = blockIdx.x;
   const int64_t t_begin = p.T * b / G, t_end = p.T * (b + 1) / G;
 
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < kMaxStages; ++i) {
-      mbar_init(&full[i], 1);
-      mbar_init(&empty[i], p.regime == 0 ? 1u : uint32_t(kWarps / p.groups));
+  if (threadIdx.x < kMaxStages) {
+    mbar_init(&full[threadIdx.x], 1);
+    mbar_init(&empty[threadIdx.x], p.regime == 0 ? 1u : uint32_t(kWarps / p.groups));
+    if (threadIdx.x < 2) {
+      mbar_init(&ms.full[threadIdx.x], 1);
+      mbar_init(&ms.done[threadIdx.x], uint32_t(kWarps));
     }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&ms.full[i], 1);
-      mbar_init(&ms.done[i], uint32_t(kWarps));
-    }
-    *abort = 0;
+    if (threadIdx.x == 0) *abort = 0;
     fence_barrier_init();
   }
   __syncthreads();
