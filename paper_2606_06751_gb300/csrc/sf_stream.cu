@@ -682,7 +682,7 @@ cudaError_t launch_stream_pass(const StreamJob& j, cudaStream_t stream) {
     const int64_t r0_rows = r0_stage_bytes(kind, j.S) / kRowBytes;
     p.regime = box_for(RS) <= r0_rows ? 0 : 1;
     p.m_rows = gain ? (j.T + j.W - 1) / j.W * RS / 16 : 0;
-    if (p.m_rows >= 1 && p.regime == 1) plan_medians(p, static_cast<int>(box_for(RS)));
+    if (p.m_rows >= 1 && p.regime == 1 && j.T >= int64_t(sms) * 4) plan_medians(p, static_cast<int>(box_for(RS)));
     p.ring_bytes = gain && p.regime == 1 ? kGainBytes : kRingBytes;
     if (p.regime == 0) {
       // whole steps per tile: as many as fit, fewer where that would leave warps without a tile
@@ -706,6 +706,7 @@ cudaError_t launch_stream_pass(const StreamJob& j, cudaStream_t stream) {
       const int64_t kb = 1024, step_bytes = RS * 8;
       if (!gain) p.groups = step_bytes <= 64 * kb ? 4 : step_bytes <= 128 * kb ? 2 : 1;
       else p.groups = step_bytes <= 32 * kb ? 4 : step_bytes <= 128 * kb ? 2 : 1;
+      while (p.groups > 1 && (p.groups - 1) * int64_t(sms) >= j.T) p.groups /= 2;  // a group for every step of a CTA
       const int64_t threads = warps * 32 / p.groups;  // of a group
       // tiles that leave each group three stages
       const int64_t ring = p.ring_bytes - p.m_slots * p.m_bytes;

@@ -382,6 +382,31 @@ def check_evidence(sf, d_np, W, options, place=dev):
             assert [[int(w[2 * i]) | int(w[2 * i + 1]) << 64 for i in range(3)] for w in got] == q
 
 
+def check_passes(sf, d_np, W):
+    d, st = dev(d_np), sf.new_status("cuda")
+    b, ob = sf.sf_window_baselines(d, W, status=st), O.baselines(d_np, W)
+    s2 = host(b.SUM.view(torch.int64)).astype(object) & ((1 << 64) - 1)
+    assert (s2[..., 0] + (s2[..., 1] << 64) == ob.SUM).all()
+    assert np.array_equal(host(b.M), ob.M) and np.array_equal(host(b.SLOW), ob.SLOW)
+    assert np.array_equal(host(b.RANK0), ob.RANK0)
+    f, o = sf.sf_frontier(d, status=st), O.frontier(d_np)
+    assert np.array_equal(host(f.a), o.a) and np.array_equal(host(f.lead), o.lead)
+    assert np.array_equal(host(f.makespan), o.makespan) and int(st.item()) == 0
+    g, ow = sf.sf_window_aggregate(d, W, status=st), O.windows(d_np, W)
+    assert np.array_equal(host(g.X), ow.X) and np.array_equal(host(g.D), ow.D)
+    assert np.array_equal(host(g.E), ow.E) and np.array_equal(host(g.C), ow.C) and int(st.item()) == 0
+
+
+# fewer steps than a CTA has warp groups for, medians beside the tiles
+@pytest.mark.parametrize("T,R,S,W", [(100, 1024, 8, 30), (153, 1024, 8, 153), (303, 700, 6, 7), (455, 641, 5, 100),
+                                     (607, 600, 8, 100), (608, 600, 8, 100)])
+@pytest.mark.parametrize("kind", ["ms", "long"])
+def test_few_steps(sf, T, R, S, W, kind):
+    d_np = durations(T, R, S, kind, T + R)
+    check_evidence(sf, d_np, W, [(None, -1), (d_np.sum(axis=2) + 1000, S - 1)])
+    check_passes(sf, d_np, W)
+
+
 # steps enough for a lane per (step, stage): every scan depth, one to 16 steps a tile, a
 # partial last tile and window, steps past 32 bits, sums past 64
 LANES = [(20000, 3, 1, 999), (9001, 60, 2, 500), (6000, 7, 6, 250), (4000, 33, 13, 300), (3000, 100, 16, 3000),
@@ -400,15 +425,7 @@ def test_step_lanes(sf, T, R, S, W, kind):
     rng = np.random.default_rng(T)
     wall = d_np.sum(axis=2) + rng.integers(-100000, 100000, size=(T, R))
     check_evidence(sf, d_np, W, [(None, -1), (wall, -1), (wall, S - 1), (None, S // 2)])
-    d, st = dev(d_np), sf.new_status("cuda")
-    b, ob = sf.sf_window_baselines(d, W, status=st), O.baselines(d_np, W)
-    s2 = host(b.SUM.view(torch.int64)).astype(object) & ((1 << 64) - 1)
-    assert (s2[..., 0] + (s2[..., 1] << 64) == ob.SUM).all()
-    assert np.array_equal(host(b.M), ob.M) and np.array_equal(host(b.SLOW), ob.SLOW)
-    assert np.array_equal(host(b.RANK0), ob.RANK0)
-    f, o = sf.sf_frontier(d, status=st), O.frontier(d_np)
-    assert np.array_equal(host(f.a), o.a) and np.array_equal(host(f.lead), o.lead)
-    assert np.array_equal(host(f.makespan), o.makespan) and int(st.item()) == 0
+    check_passes(sf, d_np, W)
 
 
 # medians that are only 8-byte aligned: steps of many and of few ranks, few steps and many
