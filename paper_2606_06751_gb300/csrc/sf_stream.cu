@@ -575,6 +575,15 @@ bool use_step_lanes(int kind, int64_t T, int64_t R, int64_t S, bool fast, int sm
   }
 }
 
+// A CTA per step (stream_generic_kernel) instead of tiles: few small steps that are not
+// whole 128-byte rows, whose tiles' barriers, copies and patched rows cost more than
+// plain loads (us, tiles / CTAs: frontier 100 x 614 x 4 6.2 / 4.1, 200 x 171 x 5
+// 6.2 / 4.1, 450 x 614 x 1 6.2 / 4.1, 620 x 614 x 1 6.2 / 6.2; evidence 152 x 1000 x 1
+// 12.5 / 8.2; baselines 200 x 171 x 12 8.2 / 10.3).
+bool use_step_ctas(int kind, int64_t T, int64_t R, int64_t S, bool whole, int sms) {
+  return !whole && R * S * 8 <= 20 * 1024 && T <= int64_t(sms) * (S <= 4 ? 3 : 2) && (kind == kFrontier || S <= 8);
+}
+
 // Whether the evidence pass keeps whole windows of medians (`rows` 128-byte
 // rows each) in shared memory, and how.  Two slots let a window's copy run
 // under the steps of the one before; one slot stands idle for a copy at each
@@ -669,11 +678,11 @@ cudaError_t launch_stream_pass(const StreamJob& j, cudaStream_t stream) {
     count_launch();
     return launch_step_lanes(kind, p, stream, j.after_clear);
   }
-  if (fast) {
+  const bool whole = RS % 16 == 0 && j.S % 2 == 0;
+  if (fast && !use_step_ctas(kind, j.T, j.R, j.S, whole, sms)) {
     const bool gain = j.gain;
     const int warps = consumer_warps(kind, j.S);
     // elements a tile may hold before its first one, in the 128-byte row both share
-    const bool whole = RS % 16 == 0 && j.S % 2 == 0;
     const int64_t pad = whole ? 0 : 15;
     p.rows = rows;
     auto box_for = [&](int64_t elems) { return (pad + elems + 15) / 16; };

@@ -397,8 +397,11 @@ def check_passes(sf, d_np, W):
     assert np.array_equal(host(g.E), ow.E) and np.array_equal(host(g.C), ow.C) and int(st.item()) == 0
 
 
-# fewer steps than a CTA has warp groups for, medians beside the tiles
-@pytest.mark.parametrize("T,R,S,W", [(100, 1024, 8, 30), (153, 1024, 8, 153), (303, 700, 6, 7), (455, 641, 5, 100),
+# few steps that are not whole 128-byte rows: a CTA per step up to 20 KB and 304 or 456
+# steps, tiles above; fewer steps than a CTA has warp groups for, medians beside the tiles
+@pytest.mark.parametrize("T,R,S,W", [(456, 640, 4, 100), (457, 640, 4, 100), (304, 319, 8, 304), (305, 319, 8, 100),
+                                     (10, 2560, 1, 4), (10, 2561, 1, 4), (200, 171, 12, 50), (304, 285, 9, 100),
+                                     (100, 1024, 8, 30), (153, 1024, 8, 153), (303, 700, 6, 7), (455, 641, 5, 100),
                                      (607, 600, 8, 100), (608, 600, 8, 100)])
 @pytest.mark.parametrize("kind", ["ms", "long"])
 def test_few_steps(sf, T, R, S, W, kind):
