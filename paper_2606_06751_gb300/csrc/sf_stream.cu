@@ -538,7 +538,15 @@ namespace {
 // the same times 64:
 //   frontier              48000 x 16 x 6    26.7 / 12.4 (26.7 / 20.5)
 //                         48000 x 48 x 6    32.8 / 32.4 (33.0 / 51)
-//   baselines             48000 x 64 x 8      62 / 46   (62 / 79)
+//                         60000 x 97 x 1    22.6 / 16.4 (22.6 / 16.4)
+//                         60000 x 129 x 2   33.7 / 37.6 (33.5 / 54)
+//                         60000 x 97 x 4    45.1 / 47.0 (45.2 / 67)
+//   with window sums      60000 x 65 x 2    39.1 / 18.5 (39.2 / 24.6)
+//                         60000 x 97 x 3    49.2 / 38.1 (49.2 / 53)
+//                         60000 x 193 x 2     55 / 58   (55 / 86)
+//   baselines             60000 x 97 x 3      54 / 37   (54 / 51)
+//                         60000 x 193 x 4     86 / 87   (86 / 123)
+//                         48000 x 64 x 8      62 / 46   (62 / 79)
 //                         24000 x 64 x 16     53 / 46   (53 / 84)
 //                         24000 x 48 x 12   39.5 / 36.8 (39.2 / 66)
 //   evidence              24000 x 64 x 16     93 / 55   (97 / 109)
@@ -556,7 +564,7 @@ namespace {
 //   medians only 8-byte   10000 x 64 x 6    22.5 / 14.5 (22.6 / 30.8)
 //   aligned               5000 x 64 x 4     12.4 / 10.3 (12.3 / 16.5)
 //                         20000 x 64 x 6      40 / 54   (40 / 111), with quality sums
-bool use_step_lanes(int kind, int64_t T, int64_t R, int64_t S, bool fast, int sms) {
+bool use_step_lanes(int kind, bool windows, int64_t T, int64_t R, int64_t S, bool fast, int sms) {
   const int64_t tiles = (T + 32 / S - 1) / (32 / S);
   if (tiles < int64_t(sms) * 4) return false;
   if (S > 16) {  // against a CTA per step
@@ -568,8 +576,11 @@ bool use_step_lanes(int kind, int64_t T, int64_t R, int64_t S, bool fast, int sm
     return T >= int64_t(sms) * 32 && tiles >= int64_t(sms) * 8 && (kind != kGainQuality || S == 16 || R <= 16);
   const bool full = S <= 4 || S == 8 || S == 16;  // few or none of the lanes idle
   switch (kind) {
-    case kFrontier: return lanes_groups(R, S) == 0 && R <= (S <= 8 ? 48 : 32) && R * S * 8 <= 3072;
-    case kBase: return R <= (S <= 8 ? 64 : S <= 11 || S == 16 ? 48 : 32);
+    case kFrontier:
+      if (lanes_groups(R, S) != 0) return false;
+      if (S <= 4) return R <= (S == 1 ? (windows ? 192 : 128) : S == 2 ? (windows ? 128 : 96) : windows ? 100 : 64);
+      return R <= (S <= 8 ? 48 : 32) && R * S * 8 <= 3072;
+    case kBase: return R <= (S == 1 ? 192 : S <= 3 ? 128 : S == 4 ? 100 : S <= 8 ? 64 : S <= 11 || S == 16 ? 48 : 32);
     case kGain: return R <= (S == 16 ? 128 : full ? 64 : S <= 11 ? 48 : 32);
     default: return R <= 16 || (R <= 48 && full && tiles >= int64_t(sms) * 16);
   }
@@ -674,7 +685,7 @@ cudaError_t launch_stream_pass(const StreamJob& j, cudaStream_t stream) {
     return e;
   }
   const int kind = j.gain ? (j.quality ? kGainQuality : kGain) : j.base ? kBase : kFrontier;
-  if (use_step_lanes(kind, j.T, j.R, j.S, fast, sms)) {
+  if (use_step_lanes(kind, j.X != nullptr, j.T, j.R, j.S, fast, sms)) {
     count_launch();
     return launch_step_lanes(kind, p, stream, j.after_clear);
   }
