@@ -8,10 +8,9 @@
 // increments a[t,.] of the frontier pass (their prefix over s), every thread
 // counts, per stage, its rank rows whose prefix equals it, and the counts are
 // summed.  Three splits of the work, chosen by launch_frontier_ties:
-//   ties_warp_kernel - up to kTieWarpRanks ranks and enough steps to fill the
-//     chip with warps: a warp per step, no CTA barrier.  Three barriers a step
-//     bound small steps (100000 x 128 x 8: 344 us with a CTA per step, 136 us,
-//     90 % of the measured copy rate, with a warp);
+//   ties_warp_kernel - a warp per step, no CTA barrier, for small steps that are
+//     many enough.  Three barriers a step bound them (100000 x 128 x 8: 344 us with a
+//     CTA per step, 136 us, 90 % of the measured copy rate, with a warp);
 //   ties_kernel      - a CTA per step, the CTA walking a range of steps; with
 //     fewer steps than the chip holds CTAs, a thread-block cluster per step,
 //     its CTAs' counts summed through distributed shared memory (one step of
@@ -32,10 +31,21 @@ namespace {
 
 constexpr int kTieThreads = 256;
 constexpr int kTieWarps = kTieThreads / 32;
-constexpr int64_t kTieWarpRanks = 512;
 constexpr int kTieCluster = 8;
-// ties_kernel CTAs per SM
-constexpr int tie_ctas(int smax) { return smax == 16 ? 2 : 4; }
+
+// Resident ties_kernel CTAs per SM.
+__host__ __device__ constexpr int tie_ctas(int smax, bool staged) { return smax <= 8 ? 4 : smax == 32 ? 1 : staged ? 2 : 3; }
+
+// Whether a step takes a warp.  A lane walks R / 32 rows alone, so the longer that is
+// the more warps per SM it takes to beat a CTA per step (us, CTA / warp: 600 x 100 x 3
+// 4.2 / 6.2, 800 x 100 x 3 6.2 / 6.2, 2500 x 100 x 3 8.2 / 6.2; 1200 x 330 x 6 8.3 / 10.3, 2500 x 330 x 6
+// 12.4 / 10.3; 1200 x 330 x 14 14.4 / 12.3; 2500 x 500 x 20 73.9 / 85.8).
+bool use_warps(int64_t T, int64_t R, int64_t S, int64_t sms) {
+  if (R <= 32) return true;
+  if (R <= 128) return T >= sms * 4;
+  if (S > 16) return R <= 340 && T >= sms * 5;
+  return R <= 512 && T >= sms * (S <= 8 ? 12 : 5);
+}
 
 __device__ __forceinline__ uint32_t hi32(int64_t v) {
   return static_cast<uint32_t>(static_cast<uint64_t>(v) >> 32);
@@ -57,11 +67,11 @@ __device__ __forceinline__ int64_t lane_frontier(const int64_t* a, int64_t t, in
 // 9 to 16 stages a row's loads are all issued before its first use (50000 x 1024 x
 // 10: 1100 -> 846 us); shorter rows gain nothing by it, longer ones cost too many
 // registers (1000 x 24: 141 against 189 us).
-template <int SMAX, bool VEC>
+template <int SMAX, bool VEC, bool STAGED = SMAX == 16>
 __device__ __forceinline__ void count_rows(const int64_t* dt, int S, int r0, int r1, int stride,
                                            const int64_t (&F)[SMAX], uint32_t (&cnt)[SMAX], uint32_t& dor,
                                            uint32_t& tor) {
-  constexpr int kStage = SMAX == 16 ? SMAX : VEC ? 2 : 1;  // stages loaded together
+  constexpr int kStage = STAGED ? SMAX : VEC ? 2 : 1;  // stages loaded together
   for (int r = r0; r < r1; r += stride) {
     const int64_t* row = dt + int64_t(r) * S;
     int64_t P = 0;
@@ -123,18 +133,18 @@ __global__ void __launch_bounds__(kTieThreads)
   if (lane == 0) report(status, bits);
 }
 
-// A cluster of CTAs per step (of one CTA in most launches), each counting an
-// equal share of the ranks.
-template <int SMAX, bool VEC>
-__global__ void __launch_bounds__(kTieThreads, SMAX <= 8 ? 4 : 2)
+// A CTA per step or, with SPLIT, a cluster of CTAs, each counting an equal share of
+// the ranks.
+template <int SMAX, bool VEC, bool SPLIT, bool STAGED = SMAX == 16>
+__global__ void __launch_bounds__(kTieThreads, tie_ctas(SMAX, STAGED))
     ties_kernel(const int64_t* __restrict__ d, int64_t T, int R, int S, const int64_t* __restrict__ a,
                 int32_t* __restrict__ ties, uint32_t* status) {
   namespace cg = cooperative_groups;
-  cg::cluster_group cluster = cg::this_cluster();
   __shared__ int64_t sF[32];
   __shared__ uint32_t wcnt[kTieWarps][32];
   __shared__ uint32_t sum[32];
-  const int csize = static_cast<int>(cluster.num_blocks()), part = static_cast<int>(cluster.block_rank());
+  const int csize = SPLIT ? static_cast<int>(cg::this_cluster().num_blocks()) : 1;
+  const int part = SPLIT ? static_cast<int>(cg::this_cluster().block_rank()) : 0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t NB = gridDim.x / csize, b = blockIdx.x / csize;
   const int64_t t_begin = T * b / NB, t_end = T * (b + 1) / NB;
@@ -154,7 +164,7 @@ __global__ void __launch_bounds__(kTieThreads, SMAX <= 8 ? 4 : 2)
       F[s] = sF[s];
       cnt[s] = 0;
     }
-    count_rows<SMAX, VEC>(d + t * R * S, S, r0 + static_cast<int>(threadIdx.x), r1, kTieThreads, F, cnt, dor, tor);
+    count_rows<SMAX, VEC, STAGED>(d + t * R * S, S, r0 + static_cast<int>(threadIdx.x), r1, kTieThreads, F, cnt, dor, tor);
 #pragma unroll
     for (int s = 0; s < SMAX; ++s) {
       if (s >= S) break;
@@ -168,7 +178,8 @@ __global__ void __launch_bounds__(kTieThreads, SMAX <= 8 ? 4 : 2)
       for (int w = 0; w < kTieWarps; ++w) c += wcnt[w][lane];
       sum[lane] = c;
     }
-    if (csize > 1) {
+    if constexpr (SPLIT) {
+      cg::cluster_group cluster = cg::this_cluster();
       cluster.sync();  // every CTA's counts are written
       if (part == 0 && warp == 0 && lane < S)
         for (int q = 1; q < csize; ++q) c += *cluster.map_shared_rank(&sum[lane], static_cast<unsigned>(q));
@@ -190,15 +201,30 @@ cudaError_t launch_frontier_ties(const int64_t* d, int64_t T, int64_t R, int64_t
   auto go = [&](auto smax, auto vec) {
     constexpr int SM = decltype(smax)::value;
     constexpr bool V = decltype(vec)::value;
-    const int64_t ctas = int64_t(sm_count()) * tie_ctas(SM);
-    if (R <= kTieWarpRanks && (T >= ctas || R <= 64)) {
-      const int grid = static_cast<int>(std::min<int64_t>(int64_t(sm_count()) * 8, (T + kTieWarps - 1) / kTieWarps));
+    const int64_t sms = sm_count();
+    if (use_warps(T, R, S, sms)) {
+      const int grid = static_cast<int>(std::min<int64_t>(sms * 8, (T + kTieWarps - 1) / kTieWarps));
       ties_warp_kernel<SM, V><<<grid, kTieThreads, 0, stream>>>(d, T, r, s, a, ties, status);
       return cudaGetLastError();
     }
-    // few steps: CTAs of a cluster share one, each with at least two rows a thread
+    // few large steps: CTAs of a cluster share one, each with at least two rows a thread
+    // (100 x 1064 x 2 4.2 us in one CTA, 6.2 in two; 100 x 4217 x 6 12.3 / 8.3)
+    const int64_t ctas = sms * (SM <= 8 ? 4 : 2);
     unsigned csize = 1;
-    while (csize < kTieCluster && T * csize * 2 <= ctas && R >= int64_t(csize) * 4 * kTieThreads) csize *= 2;
+    if (R * S * 8 >= 72 * 1024)
+      while (csize < kTieCluster && T * csize * 2 <= ctas && R >= int64_t(csize) * 4 * kTieThreads) csize *= 2;
+    if (csize == 1) {
+      // staged rows hold two CTAs per SM: a few more steps than those run in one round
+      // of three without (330 x 1064 x 14 14.3 us staged, 12.3 not; 600 x 1064 x 14 14.4, 20.5)
+      if constexpr (SM == 16)
+        if (T > ctas && T <= sms * tie_ctas(SM, false)) {
+          ties_kernel<SM, V, false, false><<<static_cast<unsigned>(T), kTieThreads, 0, stream>>>(d, T, r, s, a, ties, status);
+          return cudaGetLastError();
+        }
+      const int grid = static_cast<int>(std::min<int64_t>(SM == 32 ? sms * 4 : ctas, T));
+      ties_kernel<SM, V, false><<<grid, kTieThreads, 0, stream>>>(d, T, r, s, a, ties, status);
+      return cudaGetLastError();
+    }
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = csize;
@@ -210,7 +236,7 @@ cudaError_t launch_frontier_ties(const int64_t* d, int64_t T, int64_t R, int64_t
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, ties_kernel<SM, V>, d, T, r, s, a, ties, status);
+    return cudaLaunchKernelEx(&cfg, ties_kernel<SM, V, true>, d, T, r, s, a, ties, status);
   };
   auto pick = [&](auto smax) {
     return S % 2 == 0 ? go(smax, std::true_type{}) : go(smax, std::false_type{});

@@ -397,6 +397,16 @@ def check_passes(sf, d_np, W):
     assert np.array_equal(host(g.E), ow.E) and np.array_equal(host(g.C), ow.C) and int(st.item()) == 0
 
 
+# either side of the lines between a warp, a CTA and a cluster of CTAs per step on 152 SMs
+@pytest.mark.parametrize("T,R,S", [(607, 33, 3), (608, 128, 9), (700, 129, 20), (759, 340, 14), (760, 340, 20),
+                                   (760, 341, 20), (760, 512, 9), (1823, 512, 8), (1824, 512, 7), (305, 600, 14),
+                                   (456, 601, 9), (457, 600, 16), (20, 1151, 8), (20, 1152, 8), (75, 2500, 16), (9, 33, 32)])
+def test_ties_forms(sf, T, R, S):
+    d_np = np.random.default_rng(T + R).integers(0, 4, size=(T, R, S)).astype(np.int64)
+    d_np[::3] += 1 << 31
+    assert np.array_equal(host(sf.sf_frontier_ties(dev(d_np))), O.frontier(d_np).ties)
+
+
 # few steps that are not whole 128-byte rows: a CTA per step up to 20 KB and 304 or 456
 # steps, tiles above; fewer steps than a CTA has warp groups for, medians beside the tiles
 @pytest.mark.parametrize("T,R,S,W", [(456, 640, 4, 100), (457, 640, 4, 100), (304, 319, 8, 304), (305, 319, 8, 100),
