@@ -251,8 +251,11 @@ __device__ __noinline__ bool clamp_column(unsigned char* row0, uint32_t swizzle_
 // The selection touches only registers and the warp's counters.  A column
 // whose median is not among the values that share row 0's high 32 bits selects
 // on 64-bit values re-read from d (all columns with an outlier past 32 bits did:
-// a heavy-tailed 50000 x 1024 x 10, W = 500, 1352 us); past 512 rows, any column
-// whose values do not share them.  Every window of a launch holds the same n rows.
+// a heavy-tailed 50000 x 1024 x 10, W = 500, 1352 us).  Past 512 rows and without
+// kFit, any column whose values do not share them does: there the loop that reads a
+// clamped column once more took 4 to 18 % of every other column (3430 x 3128 x 8,
+// W = 343, 247 -> 211 us without it; out of line 232).  Every window of a launch
+// holds the same n rows.
 //
 // Resident CTAs hide each tile's copy and selection chain, so the registers are
 // held to what the most CTAs allow without spilling the column (512-row columns,
@@ -318,7 +321,7 @@ __global__ void __launch_bounds__(kMedThreads, med_min_ctas(NPL))
     auto live = [&](int i) { return (kFit && i + 1 < NPL) || lane + 32 * i < n; };
     uint32_t xl[NPL];
     uint32_t hand, hor, live_x = 0u;
-    for (bool again = NPL <= 16 && mine;; again = false) {
+    for (bool again = NPL <= 16 && kFit && mine;; again = false) {
       hand = 0xffffffffu;
       hor = 0u;
 #pragma unroll
@@ -330,9 +333,9 @@ __global__ void __launch_bounds__(kMedThreads, med_min_ctas(NPL))
         hand &= okr ? v.y : 0xffffffffu;
         hor |= okr ? v.y : 0u;
       }
-      // a column whose high words differ is clamped and read once more (not with 32
-      // slots: the call's registers would spill them)
-      if (NPL > 16 || !again || __reduce_and_sync(kFull, hand) == __reduce_or_sync(kFull, hor) ||
+      // with kFit, a column whose high words differ is clamped and read once more (not
+      // with 32 slots: the call's registers would spill them)
+      if (NPL > 16 || !kFit || !again || __reduce_and_sync(kFull, hand) == __reduce_or_sync(kFull, hor) ||
           !clamp_column(tile, static_cast<uint32_t>(warp), n, lane))
         break;
     }
