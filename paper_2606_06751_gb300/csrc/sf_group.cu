@@ -121,8 +121,11 @@ __device__ __forceinline__ int64_t step_frontier(unsigned long long* Fk, int i, 
 // accX [G][S] i64 and accD [G] i64 (the current window's sums).  SPLIT: a cluster
 // of CTAs shares each step's ranks, and its CTAs combine their Fk through
 // distributed shared memory, each for every csize-th group.
+// Five CTAs per SM: seven and twelve stages would take registers for four, a second
+// round for 609 to 760 steps (650 x 2100 x 7 32.8 -> 24.9 us, 650 x 4500 x 12 91 -> 62).
 template <int SC, bool SPLIT>
-__global__ void __launch_bounds__(kGrThreads) group_window_kernel(const GroupParams p) {
+__global__ void __launch_bounds__(kGrThreads, (SPLIT ? SC <= 12 : SC == 7 || SC == 12) ? 5 : 0)
+    group_window_kernel(const GroupParams p) {
   namespace cg = cooperative_groups;
   extern __shared__ __align__(16) unsigned char dyn[];
   const int S = SC > 0 ? SC : static_cast<int>(p.S);
@@ -420,13 +423,13 @@ cudaError_t launch_group_t(const GroupParams& p, size_t smem, cudaStream_t strea
     cudaGetLastError();
     per_sm = 1;
   }
-  const int64_t slots = int64_t(per_sm) * sm_count();
   count_launch();
-  // few steps of many ranks: CTAs enough for every SM, at least 1024 ranks each (us, a
+  // few steps of many ranks: up to four CTAs per SM, at least 1024 ranks each (us, a
   // CTA per step / split: 1 x 8192 x 8 47 / 16, 100 x 8192 x 8 49 / 25, 250 x 8192 x 8
-  // 62 / 41, 100 x 30000 x 16 299 / 130; two CTAs for 1024 ranks, 300 x 1024 x 6 12 / 14)
+  // 62 / 41, 100 x 30000 x 16 299 / 130; two CTAs for 1024 ranks, 300 x 1024 x 6 12 / 14;
+  // more CTAs, 400 x 2100 x 8 22.6 / 30.8, eight for two, 100 x 9000 x 8 28.5 / 37.8)
   int csize = 1;
-  while (csize < 8 && p.T * csize * 2 <= slots && p.R >= int64_t(csize) * 2048) csize *= 2;
+  while (csize < 8 && p.T * csize * 2 <= int64_t(sm_count()) * 4 && p.R >= int64_t(csize) * 2048) csize *= 2;
   if (csize > 1) {
     auto split = group_window_kernel<SC, true>;
     e = cudaFuncSetAttribute(split, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -445,7 +448,7 @@ cudaError_t launch_group_t(const GroupParams& p, size_t smem, cudaStream_t strea
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, split, p);
   }
-  kern<<<static_cast<unsigned>(std::min(slots, p.T)), kGrThreads, smem, stream>>>(p);
+  kern<<<static_cast<unsigned>(std::min(int64_t(per_sm) * sm_count(), p.T)), kGrThreads, smem, stream>>>(p);
   return cudaGetLastError();
 }
 
