@@ -506,8 +506,13 @@ cudaError_t launch_column(ChipParams p, cudaStream_t stream) {
 //    stages: those take the step form (40 x 1024 x 1 13.3 / 14.4 / 7.6, 300 x 2048 x 1
 //    20.5 / 23.6 / 8.3, against 1500 x 1024 x 1 38.2 / 14.4 / 22.6).
 //  - With more stages few large steps leave SMs idle that the passes through L2 use:
-//    20 x 2048 x 10 16.4 / 20.5, 80 x 2048 x 10 22.6 / 20.6; 40 x 3000 x 6 16.4 / 20.5,
-//    300 x 3000 x 6 30.8 / 26.7.
+//    20 x 2048 x 10 16.4 / 20.5, 80 x 2048 x 10 22.6 / 20.6.
+//  - The step form's warps go round the columns of four, six, eight and nine stages with
+//    the fewest to spare, and it takes few steps of three long ones: passes / step form
+//    300 x 2050 x 4 24.6 / 14.4 (71.8 / 52.4), 330 x 4300 x 4 32.9 / 34.9 (129 / 183),
+//    300 x 2500 x 6 28.8 / 22.6 (28.8 / 26.5), 200 x 3600 x 6 28.8 / 30.8, 600 x 2500 x 8
+//    56.3 / 59.6 (62.3 / 83.4), 330 x 2500 x 9 61.7 / 74.3 (63.3 / 90.7); 10 x 7000 x 3
+//    18.6 / 22.7, 300 x 7000 x 3 69.8 / 28.7.
 enum RankForm { kRankPasses, kRankLanes, kRankWarp, kRankColumn, kRankStep };
 
 RankForm rank_form(int64_t T, int64_t R, int64_t S) {
@@ -521,7 +526,9 @@ RankForm rank_form(int64_t T, int64_t R, int64_t S) {
     if (step && (S <= 2 ? R > 256 && T < sms * 4 : S <= 4 && R > 1024 && T < sms * 2)) return kRankStep;
     return S > 8 && R > 1024 && T < sms / 2 ? kRankPasses : kRankColumn;
   }
-  return step && S != 8 && (S <= 4 || T >= sms) ? kRankStep : kRankPasses;
+  if (!step || S == 8) return kRankPasses;
+  if (S <= 4) return S <= 2 || (S == 4 ? R <= 2500 : R <= 6000 || T >= sms) ? kRankStep : kRankPasses;
+  return T >= sms && (S == 6 ? R <= 2500 : S != 9 || R <= 2250) ? kRankStep : kRankPasses;
 }
 
 }  // namespace
