@@ -63,14 +63,17 @@ __device__ __forceinline__ void load_global_row(const int64_t* src, int64_t (&v)
 // (ranks are disjoint, so the largest key still carries the lowest attaining
 // rank) and runs the step's epilogue.  No global scratch.
 //
-// Two rows in flight per thread hold half the registers of four, so that half as
-// many CTAs again are resident and steps split further: frontier, us, four rows /
-// two: 100 x 8192 x 8 14.4 / 12.4, 160 x 8192 x 8 22.5 / 18.4, 200 x 32768 x 8
-// 72.7 / 65.9.  Where four rows split a step as well and leave a CTA 8192 ranks or
-// more, they are as fast or faster (64 x 65536 x 8 44.8 / 47.4, 140 x 16384 x 8
-// 27.3 / 28.4).
+// Two rows in flight per thread hold half the registers of four, so that more CTAs
+// are resident and steps split further.  That pays where the fullest SM then holds
+// fewer ranks and a step has six stages or more, or twelve at the same number: frontier,
+// us, four rows / two: 200 x 8192 x 8 22.6 / 18.5, 100 x 8192 x 8 14.4 / 12.3,
+// 140 x 5504 x 12 13.9 / 12.3; 140 x 8192 x 8 14.4 / 16.2, 75 x 11818 x 16 30.9 / 37.6;
+// 54 x 10000 x 4 7.3 / 8.3, 54 x 14356 x 2 with window sums 8.2 / 12.3.  (Ten stages
+// gain with as many CTAs too, 140 x 3000 x 10 10.3 / 8.7.)  Where four rows split a step
+// as well and leave a CTA 5000 ranks or more, they are as fast or faster
+// (64 x 65536 x 8 44.8 / 47.4, 140 x 16384 x 8 27.3 / 28.4, 23 x 34248 x 16 37.7 / 45.2).
 constexpr int kSplitThreads = 256;
-constexpr int64_t kSplitLongShare = 8192;  // ranks of a CTA from which four rows are in flight
+constexpr int64_t kSplitLongShare = 5000;  // ranks of a CTA from which four rows are in flight
 constexpr int kSplitMaxCluster = 16;  // above 8: a non-portable cluster size, allowed per kernel
 
 template <int S, int U>
@@ -254,8 +257,13 @@ Split plan_split(const StreamJob& j, int sms) {
   q.rows = 4;
   q.csize = split_cluster<4>(S, j.T, j.R);
   if (q.csize > 1 && j.R / q.csize >= kSplitLongShare) return q;
-  q.rows = 2;
-  q.csize = split_cluster<2>(S, j.T, j.R);
+  const int more = split_cluster<2>(S, j.T, j.R);
+  auto busiest = [&](int c) { return double((j.T * c + sms - 1) / sms) * j.R / c; };  // ranks of the fullest SM
+  if (q.csize == 0 || (S == 10 && more == q.csize) ||
+      (more > q.csize && (S >= 12 ? busiest(more) <= busiest(q.csize) : S >= 6 && busiest(more) <= 0.87 * busiest(q.csize)))) {
+    q.rows = 2;
+    q.csize = more;
+  }
   return q;
 }
 

@@ -262,6 +262,14 @@ def test_split_steps(sf, T, R, S, kind):
     assert int(st.item()) == 0
 
 
+# four and two rows in flight per thread, by stages, ranks and steps
+@pytest.mark.parametrize("T,R,S", [(8, 1500, 2), (54, 1030, 4), (200, 1100, 8), (100, 8192, 8), (140, 1100, 10), (75, 2100, 12),
+                                   (45, 1501, 12), (16, 1300, 16), (4, 33000, 6), (200, 1024, 7), (130, 1050, 14)])
+@pytest.mark.parametrize("kind", ["ms", "long"])
+def test_split_rows(sf, T, R, S, kind):
+    test_split_steps(sf, T, R, S, kind)
+
+
 # every stage count of its own kernel and those without, in steps of one and two
 # rows of 256 ranks, more groups than the lanes take
 @pytest.mark.parametrize("T,R,S", [(500, r, s) for s in (2, 3, 5, 7, 9, 11, 12, 13) for r in (256, 257, 513)])
