@@ -34,7 +34,7 @@ constexpr int kTieWarps = kTieThreads / 32;
 constexpr int kTieCluster = 8;
 
 // Resident ties_kernel CTAs per SM.
-__host__ __device__ constexpr int tie_ctas(int smax, bool staged) { return smax <= 8 ? 4 : smax == 32 ? 1 : staged ? 2 : 3; }
+__host__ __device__ constexpr int tie_ctas(int smax, bool staged) { return smax <= 8 ? 4 : smax == 32 || staged ? 2 : 3; }
 
 // Whether a step takes a warp.  A lane walks R / 32 rows alone, so the longer that is
 // the more warps per SM it takes to beat a CTA per step (us, CTA / warp: 600 x 100 x 3
@@ -42,7 +42,7 @@ __host__ __device__ constexpr int tie_ctas(int smax, bool staged) { return smax 
 // 12.4 / 10.3; 1200 x 330 x 14 14.4 / 12.3; 2500 x 500 x 20 73.9 / 85.8).
 bool use_warps(int64_t T, int64_t R, int64_t S, int64_t sms) {
   if (R <= 32) return true;
-  if (R <= 128) return T >= sms * 4;
+  if (R <= 128) return T >= sms * (R > 64 && S <= 8 ? 8 : 4);
   if (S > 16) return R <= 340 && T >= sms * 5;
   return R <= 512 && T >= sms * (S <= 8 ? 12 : 5);
 }
@@ -212,7 +212,7 @@ cudaError_t launch_frontier_ties(const int64_t* d, int64_t T, int64_t R, int64_t
     const int64_t ctas = sms * (SM <= 8 ? 4 : 2);
     unsigned csize = 1;
     if (R * S * 8 >= 72 * 1024)
-      while (csize < kTieCluster && T * csize * 2 <= ctas && R >= int64_t(csize) * 4 * kTieThreads) csize *= 2;
+      while (csize < kTieCluster && T * csize * 2 <= (csize > 1 ? ctas * 7 / 8 : ctas) && R >= int64_t(csize) * 4 * kTieThreads) csize *= 2;
     if (csize == 1) {
       // staged rows hold two CTAs per SM: a few more steps than those run in one round
       // of three without (330 x 1064 x 14 14.3 us staged, 12.3 not; 600 x 1064 x 14 14.4, 20.5)
