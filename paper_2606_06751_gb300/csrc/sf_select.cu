@@ -922,26 +922,37 @@ cudaError_t launch_zero_many(const ZeroList& z, cudaStream_t stream, bool* launc
   return cudaGetLastError();
 }
 
+// Whether windows of n rows take a lane per column.  Fewer tiles than four warps per SM:
+// a warp per column spreads further (48 columns by 10 windows 4.3 against 12.3 us).
+// Otherwise by estimates of both times: the lanes pay for 32 columns where a step has
+// fewer, a warp per column for eight (us, warps / lanes: 10000 windows of 100 rows, 8
+// columns 39 / 66, 16 76 / 77, 32 146 / 82, 40 181 / 161; of 20 rows, 8 columns 33 / 19;
+// 620 windows of 128 rows, 24 columns 10.3 / 13.9).
+bool use_median_lanes(int64_t nW, int64_t RS, int64_t n, bool bulk) {
+  const int64_t tiles = nW * ((RS + 31) / 32), groups = nW * ((RS + kMedCols - 1) / kMedCols);
+  if (n > kLaneMedMaxRows || tiles < int64_t(sm_count()) * 4) return false;
+  return !bulk || 0.07 * n + tiles * 0.000075 * n < groups * 0.00365;
+}
+
 cudaError_t launch_window_median(const int64_t* d, int64_t T, int64_t R, int64_t S, int64_t W,
                                  int64_t* m, uint32_t* status, cudaStream_t stream) {
   const int64_t RS = R * S;
   const int64_t nW = (T + W - 1) / W;
   const int64_t ngroups = (RS + kMedCols - 1) / kMedCols;
   const int64_t n = std::min(W, T);
-  // (fewer tiles than four warps per SM: a warp per column spreads further, 48 columns
-  // by 10 windows 4.3 against 12.3 us)
-  if (n <= kLaneMedMaxRows && nW * ((RS + 31) / 32) >= int64_t(sm_count()) * 4) {
+  // Bulk-copy path: rows of d are 16-byte multiples (RS even), d is 16-byte
+  // aligned, windows fit the register path, the driver encoder is available.
+  // A launch's windows share one row count (the slot tests depend on it), so
+  // a short last window gets its own launch.
+  const bool bulk = RS % 2 == 0 && reinterpret_cast<uintptr_t>(d) % 16 == 0 && n <= 1024 && T < (int64_t(1) << 31) &&
+                    encode_fn() != nullptr;
+  if (use_median_lanes(nW, RS, n, bulk)) {
     if (n <= 32) return launch_median_lanes<32>(d, T, RS, W, m, stream);
     if (n <= 64) return launch_median_lanes<64>(d, T, RS, W, m, stream);
     if (n <= 104) return launch_median_lanes<104>(d, T, RS, W, m, stream);
     return launch_median_lanes<128>(d, T, RS, W, m, stream);
   }
-  // Bulk-copy path: rows of d are 16-byte multiples (RS even), d is 16-byte
-  // aligned, windows fit the register path, the driver encoder is available.
-  // A launch's windows share one row count (the slot tests depend on it), so
-  // a short last window gets its own launch.
-  if (RS % 2 == 0 && reinterpret_cast<uintptr_t>(d) % 16 == 0 && n <= 1024 && T < (int64_t(1) << 31) &&
-      encode_fn() != nullptr) {
+  if (bulk) {
     const int64_t n_last = T - (nW - 1) * W;
     const int64_t nW_first = n_last == n ? nW : nW - 1;
     bool done = false;

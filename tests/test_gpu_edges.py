@@ -110,6 +110,18 @@ def test_median_lanes(sf, T, R, S, W, kind):
     assert np.array_equal(host(sf.sf_window_median(dev(d_np), W)), O.window_median(d_np, W))
 
 
+# windows enough for a lane per column on 152 SMs: rows of each form and one more, columns
+# for one tile of lanes and two, odd counts, a short last window; and one column, row or
+# window to the other side of the lines
+@pytest.mark.parametrize("T,R,S,W", [(9800, 4, 8, 16), (9740, 3, 20, 16), (9720, 16, 2, 32), (10100, 16, 4, 33), (19500, 31, 2, 64),
+                                     (20001, 13, 5, 65), (31000, 5, 12, 100), (31650, 20, 4, 104), (32000, 19, 3, 105),
+                                     (38930, 33, 3, 128), (77900, 8, 11, 128), (9760, 11, 3, 16), (9800, 1, 7, 16), (31000, 12, 2, 50),
+                                     (31000, 10, 2, 50), (62000, 4, 4, 100), (60700, 5, 4, 100)])
+@pytest.mark.parametrize("kind", ["ms", "words", "far"])
+def test_median_lanes_many_windows(sf, T, R, S, W, kind):
+    test_median_lanes(sf, T, R, S, W, kind)
+
+
 # steps held on chip: keys per lane, per warp, the CTA form's columns in registers
 # and in shared memory, the first ranks past each, columns in which every key falls
 # into a few bins, and medians on both sides of the bracket
