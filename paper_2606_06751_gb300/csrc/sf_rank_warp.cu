@@ -146,7 +146,7 @@ __device__ __forceinline__ bool warp_step(const int64_t* dt, int R, bool of_pref
       uint32_t c = 0;
 #pragma unroll
       for (int i = 0; i < NPL; ++i) c += k[s][i] <= m ? 1u : 0u;
-      c = NPL == 1 ? static_cast<uint32_t>(__popc(__ballot_sync(kFull, c != 0))) : __reduce_add_sync(kFull, c);
+      c = __reduce_add_sync(kFull, c);
       if (lane == s) cnt = c;
     }
     if (open) {

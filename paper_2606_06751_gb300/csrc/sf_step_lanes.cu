@@ -311,7 +311,10 @@ cudaError_t launch_kind(const Params& p, cudaStream_t stream, bool pdl) {
   if (p.S <= 4) return launch_logs<KIND, 2>(p, stream, pdl);
   if (p.S <= 8) return launch_logs<KIND, 3>(p, stream, pdl);
   if (p.S <= 16) return launch_logs<KIND, 4>(p, stream, pdl);
-  return launch_logs<KIND, 5>(p, stream, pdl);
+  if constexpr (is_gain(KIND))
+    return launch_logs<KIND, 5>(p, stream, pdl);
+  else
+    return cudaErrorInvalidValue;  // use_step_lanes: only evidence takes more than 16 stages here
 }
 
 }  // namespace
