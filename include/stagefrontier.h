@@ -165,8 +165,9 @@ sf_status sf_window_baselines(const int64_t* d, int64_t T, int64_t R, int64_t S,
  * Outputs device, nullable (at least one).  workspace: device, 256-byte
  * aligned, at least one step's scratch; sf_rank_workspace_size(T, R, S)
  * bytes (about 40 MB, so that the scratch stays in L2) processes the steps
- * in the fewest chunks that still fit L2.  The workspace is overwritten and
- * may be reused as soon as the call's work on `stream` is done.
+ * in the fewest chunks that still fit L2.  The workspace is required for every
+ * shape, but steps whose selection fits on chip leave it untouched; otherwise it
+ * is overwritten.  It may be reused as soon as the call's work on `stream` is done.
  */
 sf_status sf_rank_lag(const int64_t* d, int64_t T, int64_t R, int64_t S, int64_t* L, int64_t* dL, int64_t* G,
                       void* workspace, size_t workspace_bytes, uint32_t* status, cudaStream_t stream);

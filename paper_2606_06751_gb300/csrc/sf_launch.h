@@ -87,7 +87,8 @@ cudaError_t launch_rank_select(const int64_t* d, int64_t T, int64_t R, int64_t S
                                int64_t W, int64_t* L, int64_t* dL, int64_t* G, int64_t* Lw, int64_t* Gw,
                                int64_t* spread, void* workspace, size_t ws_bytes, uint32_t* status,
                                cudaStream_t stream);
-// The same for steps that fit on chip (rank_on_chip), without the workspace.
+// The same for steps that rank_on_chip selects, which use no workspace (the entry points
+// still ask for one, whatever the form).
 bool rank_on_chip(int64_t T, int64_t R, int64_t S);
 cudaError_t launch_rank_chip(const int64_t* d, int64_t T, int64_t R, int64_t S, int of_prefix, int64_t t0, int64_t W,
                              int64_t* L, int64_t* dL, int64_t* G, int64_t* Lw, int64_t* Gw, int64_t* spread,

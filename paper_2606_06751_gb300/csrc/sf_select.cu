@@ -489,8 +489,9 @@ __global__ void __launch_bounds__(kMedThreads)
 // s*R + r for E); value 0 is not a suspect.
 //
 // A window's (stage, rank) entries are split over a cluster of one to
-// kTopCluster CTAs (top_cluster: one tile of entries each, eight at most).  Each CTA reads its slice once, kTopTile entries at a time with the
-// next tile's loads in flight, and appends the positive entries to a list in
+// kTopCluster CTAs (about one tile of entries each, eight at most).  Each CTA reads
+// its slice once, kTopTile entries at a time with the next tile's loads in flight,
+// and appends the positive entries to a list in
 // shared memory: lead-rank credit is sparse (at most one rank per step and
 // stage), so a slice's list usually ends far below its capacity.  A list that
 // could not take another whole tile is first cut to its k best.  The cut runs

@@ -19,8 +19,10 @@
 // of lanes, one step each).  A few hundred steps over many ranks split each
 // step's ranks over a thread-block cluster (split_frontier_kernel).
 //
-// Generic path (17 to 32 stages; medians that are only 8-byte aligned): plain
-// global loads, a warp or a CTA per step.  All paths share the per-step
+// Generic path (17 to 32 stages; medians that are only 8-byte aligned; few small
+// steps that are not whole 128-byte rows; tensors that no tensor map describes): a
+// CTA per step, plain global loads or, past 16 stages, a ring of bulk copies.  A lane
+// per (step, stage) takes many small steps (sf_step_lanes.cu).  All paths share the per-step
 // epilogues.  A pass that follows the clear of its own outputs starts as that
 // clear's programmatic dependent and writes only after griddep_wait().
 #include <algorithm>
@@ -809,9 +811,8 @@ cudaError_t launch_stream_pass(const StreamJob& j, cudaStream_t stream) {
     if constexpr (SM > 16) {
       // more than 16 stages: registers hold these kernels to one or two CTAs
       // per SM, and the bulk-copy ring keeps the loads off their step chain
-      // (512 x 24: 0.434 -> 0.405 ms).  Up to 16 stages four CTAs per SM
-      // hide the loads better than a ring that leaves room for three (1000 x 5:
-      // 0.229 against 0.285 ms), so those shapes read global memory.
+      // (512 x 24: 0.434 -> 0.405 ms).  Up to 16 stages these kernels see few
+      // steps, and four CTAs per SM hide the loads.
       if (chunk != 0) {
         if (j.gain) return go(stream_generic_kernel<SM, 1, false, true>, true);
         if (j.base && vec) return go(stream_generic_kernel<SM, 2, true, true>, true);

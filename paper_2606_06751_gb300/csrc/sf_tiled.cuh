@@ -14,7 +14,7 @@
 // kernels, whose swizzled addresses need no arithmetic per load).  Elements past
 // the last whole row of d are written into the tile by its readers.  Steps that
 // are not whole rows took a warp or a CTA each with plain loads before: evidence
-// pass over 4001 x 1001 x 13 572 -> 105 us, 13421 x 1000 x 5 279 -> 123 us.  The tiles are
+// pass over 4001 x 1001 x 13 572 -> 105 us, 13421 x 1000 x 5 279 -> 129 us.  The tiles are
 // 128B-swizzled for 4, 8 and 16 stages, where the 16-byte reads of consecutive
 // rank rows would share banks; for other even and for odd stage counts the
 // rows' stride already spreads them.
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__((consumer_warps(KIND, S) + kProducers) * 32, 1
   };
 
   if (p.regime == 0) {
-    // ---- each warp owns every 8th tile (K whole steps) and two ring stages
+    // ---- the warps take the tiles (K whole steps) in turn, each with two ring stages
     const int64_t n_local = t_end - t_begin;
     const int64_t n_tiles = (n_local + p.K - 1) / p.K;
     uint32_t i = 0;
