@@ -208,11 +208,15 @@ cudaError_t launch_frontier_ties(const int64_t* d, int64_t T, int64_t R, int64_t
       return cudaGetLastError();
     }
     // few large steps: CTAs of a cluster share one, each with at least two rows a thread
-    // (100 x 1064 x 2 4.2 us in one CTA, 6.2 in two; 100 x 4217 x 6 12.3 / 8.3)
+    // (100 x 1064 x 2 4.2 us in one CTA, 6.2 in two; 100 x 4217 x 6 12.3 / 8.3).  Clusters of
+    // four and more need room to be placed (152 x 8192 x 8 in four, filling every slot, 21.6
+    // us, in two 18.4; 76 x 15000 x 32 in four 137, in two 117)
     const int64_t ctas = sms * (SM <= 8 ? 4 : 2);
     unsigned csize = 1;
     if (R * S * 8 >= 72 * 1024)
-      while (csize < kTieCluster && T * csize * 2 <= (csize > 1 ? ctas * 7 / 8 : ctas) && R >= int64_t(csize) * 4 * kTieThreads) csize *= 2;
+      while (csize < kTieCluster && T * csize * 2 <= (csize > 1 ? ctas * 7 / 8 : ctas) &&
+             R >= int64_t(csize) * 4 * kTieThreads)
+        csize *= 2;
     if (csize == 1) {
       // staged rows hold two CTAs per SM: a few more steps than those run in one round
       // of three without (330 x 1064 x 14 14.3 us staged, 12.3 not; 600 x 1064 x 14 14.4, 20.5)
