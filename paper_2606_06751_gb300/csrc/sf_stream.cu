@@ -568,6 +568,18 @@ namespace {
 //   with quality sums     24000 x 16 x 10     53 / 33.8 (63 / 56)
 //                         24000 x 48 x 16    127 / 88   (127 / 164)
 //                         24000 x 32 x 12     49 / 65   (49 / 116)
+//                         100000 x 100 x 2   188 / 114  (188 / 114)
+//                         66666 x 100 x 3    143 / 114  (143 / 186)
+//                         33333 x 50 x 3      43 / 43   (43 / 69)
+//                         390625 x 64 x 4    506 / 401  (508 / 610)
+//                         83333 x 24 x 10    150 / 117  (185 / 202)
+//                         97656 x 64 x 16    546 / 428  (573 / 776)
+//                         19531 x 64 x 16    119 / 107  (127 / 205)
+//                         1790 x 15 x 32     100 / 15   (101 / 25), a CTA per step / lanes
+//                         855 x 60 x 20       39 / 25   (39 / 53)
+//                         1300 x 96 x 20      57 / 37   (57 / 84)
+//                         1300 x 128 x 24     70 / 45   (70 / 107)
+//                         1300 x 300 x 24    113 / 97   (113 / 242)
 //                         2500 x 192 x 24    131 / 90   (131 / 220)
 //                         2500 x 192 x 20    105 / 88   (105 / 214)
 //                         9000 x 192 x 20    367 / 251  (368 / 499)
@@ -580,7 +592,9 @@ bool use_step_lanes(int kind, bool windows, int64_t T, int64_t R, int64_t S, boo
   if (S > 16) {  // against a CTA per step
     if (kind == kGain) return R <= 192 || T >= int64_t(sms) * (S > 24 ? 4 : 10);
     if (kind != kGainQuality) return false;
-    return S >= 24 ? T * S >= int64_t(sms) * 384 : R <= 192 && T >= int64_t(sms) * (R <= 96 ? 10 : 30);
+    if (R <= (S < 24 ? 40 : 64)) return true;
+    if (S >= 24) return T * S >= int64_t(sms) * (R <= 96 ? 120 : R <= 128 ? 150 : 260);
+    return R <= 192 && T >= int64_t(sms) * (R <= 64 ? 5 : R <= 96 ? 8 : R <= 128 ? 11 : 50);
   }
   if (!fast)  // against a CTA per step
     return T >= int64_t(sms) * 32 && tiles >= int64_t(sms) * 8 && (kind != kGainQuality || S == 16 || R <= 16);
@@ -592,7 +606,13 @@ bool use_step_lanes(int kind, bool windows, int64_t T, int64_t R, int64_t S, boo
       return R <= (S <= 8 ? 48 : 32) && R * S * 8 <= 3072;
     case kBase: return R <= (S == 1 ? 192 : S <= 3 ? 128 : S == 4 ? 100 : S <= 8 ? 64 : S <= 11 || S == 16 ? 48 : 32);
     case kGain: return R <= (S == 16 ? 128 : full ? 64 : S <= 11 ? 48 : 32);
-    default: return R <= 16 || (R <= 48 && full && tiles >= int64_t(sms) * 16);
+    default: {
+      const int64_t per_sm = tiles / sms;
+      if (R <= 16) return true;
+      if (S >= 9 && S <= 11) return R <= 24 && per_sm >= 100;
+      const bool many = per_sm >= (S <= 2 ? 16 : S == 3 ? 32 : S == 4 ? 64 : 100);
+      return full && per_sm >= 16 && R <= (!many || S == 8 ? 48 : S == 16 ? 80 : 128);
+    }
   }
 }
 

@@ -450,7 +450,9 @@ LANES = [(20000, 3, 1, 999), (9001, 60, 2, 500), (6000, 7, 6, 250), (4000, 33, 1
          (6000, 48, 6, 333), (9800, 48, 8, 700), (2600, 48, 11, 2600), (4000, 32, 13, 300), (4000, 16, 14, 250),
          (4900, 48, 16, 500), (1530, 96, 17, 50), (4600, 97, 17, 500), (2500, 130, 24, 100),
          (20000, 128, 1, 500), (20000, 192, 1, 999), (19500, 193, 1, 500), (9800, 96, 2, 333), (9800, 128, 2, 500),
-         (6100, 128, 3, 100), (6500, 64, 4, 999), (5000, 100, 4, 500), (4900, 101, 4, 700)]
+         (6100, 128, 3, 100), (6500, 64, 4, 999), (5000, 100, 4, 500), (4900, 101, 4, 700),
+         (39000, 128, 2, 1000), (48700, 49, 3, 999), (45700, 17, 10, 5000),
+         (620, 40, 17, 100), (620, 41, 17, 100), (1000, 128, 24, 500), (1400, 200, 32, 1000)]
 
 
 @pytest.mark.parametrize("T,R,S,W", LANES)
