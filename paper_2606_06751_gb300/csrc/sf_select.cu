@@ -928,11 +928,14 @@ cudaError_t launch_zero_many(const ZeroList& z, cudaStream_t stream, bool* launc
 // Otherwise by estimates of both times: the lanes pay for 32 columns where a step has
 // fewer, a warp per column for eight (us, warps / lanes: 10000 windows of 100 rows, 8
 // columns 39 / 66, 16 76 / 77, 32 146 / 82, 40 181 / 161; of 20 rows, 8 columns 33 / 19;
-// 620 windows of 128 rows, 24 columns 10.3 / 13.9).
-bool use_median_lanes(int64_t nW, int64_t RS, int64_t n, bool bulk) {
+// 620 windows of 128 rows, 24 columns 10.3 / 13.9; 46 windows of 100 rows, 576 columns, and
+// one of 15 20.0 / 14.1).
+bool use_median_lanes(int64_t T, int64_t W, int64_t RS, bool bulk) {
+  const int64_t n = std::min(W, T), nW = (T + W - 1) / W;
   const int64_t tiles = nW * ((RS + 31) / 32), groups = nW * ((RS + kMedCols - 1) / kMedCols);
   if (n > kLaneMedMaxRows || tiles < int64_t(sm_count()) * 4) return false;
-  return !bulk || 0.07 * n + tiles * 0.000075 * n < groups * 0.00365;
+  const double last = T % W && nW > 1 ? 5.0 : 0.0;  // a short last window is a launch of its own there
+  return !bulk || 0.07 * n + tiles * 0.000075 * n < last + groups * 0.00365;
 }
 
 cudaError_t launch_window_median(const int64_t* d, int64_t T, int64_t R, int64_t S, int64_t W,
@@ -947,7 +950,7 @@ cudaError_t launch_window_median(const int64_t* d, int64_t T, int64_t R, int64_t
   // a short last window gets its own launch.
   const bool bulk = RS % 2 == 0 && reinterpret_cast<uintptr_t>(d) % 16 == 0 && n <= 1024 && T < (int64_t(1) << 31) &&
                     encode_fn() != nullptr;
-  if (use_median_lanes(nW, RS, n, bulk)) {
+  if (use_median_lanes(T, W, RS, bulk)) {
     if (n <= 32) return launch_median_lanes<32>(d, T, RS, W, m, stream);
     if (n <= 64) return launch_median_lanes<64>(d, T, RS, W, m, stream);
     if (n <= 104) return launch_median_lanes<104>(d, T, RS, W, m, stream);

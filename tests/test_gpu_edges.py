@@ -116,7 +116,7 @@ def test_median_lanes(sf, T, R, S, W, kind):
 @pytest.mark.parametrize("T,R,S,W", [(9800, 4, 8, 16), (9740, 3, 20, 16), (9720, 16, 2, 32), (10100, 16, 4, 33), (19500, 31, 2, 64),
                                      (20001, 13, 5, 65), (31000, 5, 12, 100), (31650, 20, 4, 104), (32000, 19, 3, 105),
                                      (38930, 33, 3, 128), (77900, 8, 11, 128), (9760, 11, 3, 16), (9800, 1, 7, 16), (31000, 12, 2, 50),
-                                     (31000, 10, 2, 50), (62000, 4, 4, 100), (60700, 5, 4, 100)])
+                                     (31000, 10, 2, 50), (62000, 4, 4, 100), (60700, 5, 4, 100), (4615, 72, 8, 100), (21324, 8, 16, 100)])
 @pytest.mark.parametrize("kind", ["ms", "words", "far"])
 def test_median_lanes_many_windows(sf, T, R, S, W, kind):
     test_median_lanes(sf, T, R, S, W, kind)
