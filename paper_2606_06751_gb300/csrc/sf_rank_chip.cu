@@ -501,12 +501,15 @@ cudaError_t launch_column(ChipParams p, cudaStream_t stream) {
 //  - Few steps of up to 128 ranks leave the lanes a tile or two per warp, and one past 32
 //    bits, which its warp takes again column by column, waits for nothing else: a CTA per
 //    step up to 10 steps per SM (300 x 64 x 4 14.4 / 10.3 / 6.2 (16.5 / 75.8 / 8.3),
-//    1500 x 64 x 8 57.9 / 10.3 / 12.3 (58.7 / 76.9 / 16.4)).
+//    1500 x 64 x 8 57.9 / 10.3 / 12.3 (58.7 / 76.9 / 16.4)).  Columns enough for the lanes
+//    come from fewer steps of many stages, and a column of 16 ranks is short (column form /
+//    lanes 1300 x 16 x 16 16 / 6.2 (21 / 68), 855 x 15 x 32 18.5 / 6.2 (37 / 72),
+//    855 x 60 x 32 23 / 12 (54 / 101), 855 x 96 x 24 18 / 16 (43 / 83)).
 //  - The column form has a warp per stage, too few to load few steps of many ranks and few
 //    stages: those take the step form (40 x 1024 x 1 13.3 / 14.4 / 7.6, 300 x 2048 x 1
 //    20.5 / 23.6 / 8.3, against 1500 x 1024 x 1 38.2 / 14.4 / 22.6).
 //  - With more stages few large steps leave SMs idle that the passes through L2 use:
-//    20 x 2048 x 10 16.4 / 20.5, 80 x 2048 x 10 22.6 / 20.6.
+//    20 x 2048 x 10 16.4 / 20.5, 80 x 2048 x 10 22.6 / 20.6, 57 x 1048 x 16 23.6 / 18.5 (217 / 55).
 //  - The step form's warps go round the columns of four, six, eight and nine stages with
 //    the fewest to spare, and it takes few steps of three long ones: passes / step form
 //    300 x 2050 x 4 24.6 / 14.4 (71.8 / 52.4), 330 x 4300 x 4 32.9 / 34.9 (129 / 183),
@@ -518,13 +521,16 @@ enum RankForm { kRankPasses, kRankLanes, kRankWarp, kRankColumn, kRankStep };
 RankForm rank_form(int64_t T, int64_t R, int64_t S) {
   const int64_t sms = sm_count();
   if (R <= kRankLaneMax) {
-    if (T < sms * 10) return kRankColumn;
+    const bool many = T >= sms * 10 ||
+                      (R <= 16 ? (S > 16 ? T * 3 >= sms * 10 : S >= 10 ? T >= sms * 5 : S >= 8 && T >= sms * 7)
+                               : S > 16 && (R <= 64 ? T * S >= sms * 110 : R <= 96 && T * S >= sms * 160));
+    if (!many) return kRankColumn;
     return R >= kRankWarpMin && S <= kRankWarpMaxS ? kRankWarp : kRankLanes;
   }
   const bool step = step_smem(R, S) <= kStepSmemMax;
   if (R <= kColMaxRanks && column_smem(R, S) <= kStepSmemMax) {
     if (step && (S <= 2 ? R > 256 && T < sms * 4 : S <= 4 && R > 1024 && T < sms * 2)) return kRankStep;
-    return S > 8 && R > 1024 && T < sms / 2 ? kRankPasses : kRankColumn;
+    return S > 8 && R > 1250 && T < sms / 2 ? kRankPasses : kRankColumn;
   }
   if (!step || S == 8) return kRankPasses;
   if (S <= 4) return S <= 2 || (S == 4 ? R <= 2500 : R <= 6000 || T >= sms) ? kRankStep : kRankPasses;

@@ -154,10 +154,11 @@ def test_rank_on_chip(sf, T, R, S, kind):
                                    (1600, 33, 17), (1600, 64, 9), (1600, 65, 16), (1600, 65, 8), (1600, 104, 10),
                                    (1530, 105, 32), (1600, 128, 8), (1600, 128, 9), (1600, 100, 5),
                                    (607, 300, 2), (608, 300, 2), (303, 1025, 3), (304, 1025, 3), (310, 2048, 4),
-                                   (700, 1500, 1), (75, 1100, 9), (76, 2048, 9), (7, 2048, 7), (20, 1100, 6),
+                                   (700, 1500, 1), (75, 1250, 9), (75, 1251, 9), (76, 2048, 9), (7, 2048, 7), (20, 1100, 6),
                                    (151, 2500, 6), (152, 2500, 6), (152, 2501, 6), (153, 2050, 11), (10, 2500, 4),
                                    (310, 2501, 4), (151, 6001, 3), (152, 6001, 3), (9, 6000, 3), (152, 2250, 9),
-                                   (152, 2251, 9)])
+                                   (152, 2251, 9), (759, 16, 10), (760, 16, 10), (1064, 13, 8), (506, 9, 17), (507, 16, 17),
+                                   (835, 64, 20), (836, 64, 20), (761, 96, 32)])
 @pytest.mark.parametrize("kind", ["ms", "long", "far", "tail", "halves"])
 def test_rank_forms(sf, T, R, S, kind):
     test_rank_on_chip(sf, T, R, S, kind)
