@@ -73,17 +73,19 @@ struct IngestTiles {
 // Steps a CTA has little to do for, and tiles for every SM (us, directly / tiles:
 // 100000 x 16 x 8 102.6 / 44.8, 100000 x 31 x 7 160 / 90, 20000 x 64 x 5 53.5 / 27.3;
 // 1500 x 32 x 6, of 94 tiles, 4.1 / 6.2; 3000 x 120 x 3, of 188, 8.2 / 10.3; 4000 x 40 x 7, of
-// 250, 10.3 / 8.2; 3000 x 4 x 1 6.2 / 4.1).  Odd stage counts, moved 8 bytes at a time
-// directly, gain up to 3 KB a step; even ones, moved 16 bytes, up to 2.5 KB and 64 ranks
-// (100000 x 64 x 4 117 / 101, 96 x 4 130 / 150, 32 x 12 125 / 122, 128 x 2 117 / 143).
+// 250, 10.3 / 8.2; 3000 x 4 x 1 6.2 / 4.1; 5000 x 128 x 1 8.2 / 10.3, 24000 26.7 / 22.6).  Odd
+// stage counts, moved 8 bytes at a time directly, gain up to 3 KB a step; even ones, moved
+// 16 bytes, up to 2.5 KB and 64 ranks (100000 x 64 x 4 117 / 101, 96 x 4 130 / 150, 32 x 12
+// 125 / 122, 128 x 2 117 / 143).
 IngestTiles plan_tiles(int64_t T, int64_t R, int64_t S, int64_t N) {
   IngestTiles p;
-  const bool small = S % 2 == 0 ? R <= 64 && R * S <= 320 : R <= (S == 1 ? 96 : 128) && R * S <= 384;
+  const bool small = S % 2 == 0 ? R <= 64 && R * S <= 320 : R <= 128 && R * S <= 384;
   if (N < kTileSteps || !small) return p;
   // even shares of the ranks (100000 x 64 x 6, whose tiles hold 63 ranks: 63 and 1 206 us, 32 and 32 125)
   const int64_t most = kTileBytes / (8 * tile_pitch(static_cast<int>(S))), blocks = (R + most - 1) / most;
   p.count = (T + N - 1) / N * ((N + kTileSteps - 1) / kTileSteps) * blocks;
-  if (2 * p.count >= sm_count() * (R * S <= 64 ? 2 : 3)) p.ranks = static_cast<int>((R + blocks - 1) / blocks);
+  const int halves = R * S <= 64 ? 2 : S == 1 && R > 96 ? 10 : 3;  // half tiles per SM
+  if (2 * p.count >= sm_count() * halves) p.ranks = static_cast<int>((R + blocks - 1) / blocks);
   return p;
 }
 

@@ -249,7 +249,7 @@ def test_gathered_tiles(sf, T, R, S, N):
 # tiles and the next ones, ranks in one tile and in equal and unequal shares of two
 @pytest.mark.parametrize("T,R,S,N", [(2432, 5, 4, 16), (2416, 5, 4, 16), (3648, 16, 8, 16), (3632, 16, 8, 16), (2600, 31, 7, 17),
                                      (5000, 64, 4, 100), (5000, 65, 4, 100), (4000, 40, 8, 33), (4000, 42, 8, 33),
-                                     (3001, 96, 1, 50), (3001, 97, 1, 50), (2600, 127, 3, 40), (2600, 128, 3, 40),
+                                     (3700, 96, 1, 50), (9600, 97, 1, 50), (12200, 128, 1, 500), (2600, 127, 3, 40), (2600, 128, 3, 40),
                                      (2600, 129, 3, 40), (3100, 10, 32, 40), (5000, 53, 6, 500), (2500, 3, 3, 1 << 40)])
 def test_gathered_tiles_everywhere(sf, T, R, S, N):
     test_gathered_tiles(sf, T, R, S, N)
